@@ -300,21 +300,25 @@ rt_status rt_set_params(rt_ctx* ctx, const void* table, const float* brdf_w, con
                                     guide_shift(ctx->cfg.env_w), s));
   if (st == RT_OK) st = cuda_status(launch_repack_bf16(ctx->wpack, ctx->wbf16, s));
   if (st != RT_OK) return st;
-  // host copy of the output layers for the BF16 kernel's parameters
-  static thread_local float host[WPACK_FLOATS];
-  if (cudaMemcpyAsync(host, ctx->wpack, sizeof(host), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+  // Host copy of the output layers for the BF16 kernel's parameters: the two spans of the packed image that hold
+  // them (I's W3 and b3; B's W3 and b3) as two rows of one strided copy, 4 KB instead of the image's 61.
+  constexpr int kSpan = WPACK_FLOATS - OFF_BW3;
+  static_assert(OFF_IB3 + 2 - OFF_IW3 <= kSpan && OFF_IW3 + kSpan <= OFF_BW3, "I's output layer lies in the first row");
+  float host[2][kSpan];
+  if (cudaMemcpy2DAsync(host, sizeof(host[0]), ctx->wpack + OFF_IW3, (OFF_BW3 - OFF_IW3) * sizeof(float), sizeof(host[0]), 2,
+                        cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return RT_ERR_CUDA;
   HeadParams& h = ctx->head;
   for (int i = 0; i < 64; ++i) {
-    h.iw3[i][0] = host[OFF_IW3 + 2 * i];
-    h.iw3[i][1] = host[OFF_IW3 + 2 * i + 1];
-    h.iw3v[i] = host[OFF_IW3 + 2 * i];
-    for (int o = 0; o < 8; ++o) h.bw3[i][o] = host[OFF_BW3 + 8 * i + o];
+    h.iw3[i][0] = host[0][2 * i];
+    h.iw3[i][1] = host[0][2 * i + 1];
+    h.iw3v[i] = host[0][2 * i];
+    for (int o = 0; o < 8; ++o) h.bw3[i][o] = host[1][8 * i + o];
   }
-  h.ib3[0] = host[OFF_IB3];
-  h.ib3[1] = host[OFF_IB3 + 1];
-  for (int o = 0; o < 8; ++o) h.bb3[o] = host[OFF_BB3 + o];
+  h.ib3[0] = host[0][OFF_IB3 - OFF_IW3];
+  h.ib3[1] = host[0][OFF_IB3 - OFF_IW3 + 1];
+  for (int o = 0; o < 8; ++o) h.bb3[o] = host[1][OFF_BB3 - OFF_BW3 + o];
   ctx->ready = true;
   return RT_OK;
 }

@@ -7,72 +7,117 @@
 // correctly rounded division by the total, and the last entry set to 1.
 // Cutpoint tables over each CDF then start the sampler's bisection close to
 // its answer.
+//
+// The running sums bound this set-up: float32 additions in index order are one
+// dependent chain, 4 cycles per texel, and nothing may reorder them.  So only
+// the chain is serial: a CTA per row loads the row's texels coalesced and forms
+// their luminances in shared memory, one thread runs the chain over it 16
+// texels at a time (the next 16 are read while these are added), and all
+// threads divide, write the row and answer its cutpoints from shared memory.
+// With the chain in global memory (one thread per row, a dependent load and a
+// strided store per texel) a 256 x 512 map took 403 us and its marginal 34 us.
 #include "mis.cuh"
 
 namespace rtk {
 namespace {
 
-__global__ void env_cdf_rows_kernel(const float4* __restrict__ env, int H, int W, float* __restrict__ cdf_m,
-                                    float* __restrict__ cdf_c) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= H) return;
-  float* row = cdf_c + (size_t)r * (W + 1);
+constexpr int kCdfThreads = 128;
+
+// v[0..n) -> its running sums, in index order, each rounded to float32; the last one is the total.
+__device__ __forceinline__ void running_sum(float* v, int n) {
   float s = 0.0f;
-  row[0] = 0.0f;
-  for (int c = 0; c < W; ++c) {
+  float4* v4 = reinterpret_cast<float4*>(v);
+  const int blocks = n / 16;
+  float4 a[4];
+  if (blocks > 0)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k] = v4[k];
+  for (int b = 0; b < blocks; ++b) {
+    float4 nx[4];
+    const int nb = min(b + 1, blocks - 1);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) nx[k] = v4[4 * nb + k];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      a[k].x = s = __fadd_rn(s, a[k].x);
+      a[k].y = s = __fadd_rn(s, a[k].y);
+      a[k].z = s = __fadd_rn(s, a[k].z);
+      a[k].w = s = __fadd_rn(s, a[k].w);
+      v4[4 * b + k] = a[k];
+      a[k] = nx[k];
+    }
+  }
+  for (int c = 16 * blocks; c < n; ++c) v[c] = s = __fadd_rn(s, v[c]);
+}
+
+// Turn the running sums v[0..n) into the CDF cdf[0..n] (0 first, 1 last) and answer its cutpoint table:
+// entry j is the bisection's answer for u = j / 2^shift (exact in float32).
+__device__ __forceinline__ void finish_cdf(float* v, int n, float* __restrict__ cdf, int* __restrict__ guide,
+                                           int shift) {
+  const float total = v[n - 1];
+  __syncthreads();   // every thread has read the total
+  for (int c = threadIdx.x; c < n; c += kCdfThreads) {
+    const float q = c + 1 < n ? __fdiv_rn(v[c], total) : 1.0f;
+    v[c] = q;
+    cdf[c + 1] = q;
+  }
+  if (threadIdx.x == 0) cdf[0] = 0.0f;
+  __syncthreads();
+  const int G = 1 << shift;
+  for (int j = threadIdx.x; j < G; j += kCdfThreads) {
+    const float u = (float)j * (1.0f / (float)G);
+    int lo = 0, hi = n;   // bisection with cdf[k] = v[k - 1] for k >= 1
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (v[mid - 1] <= u) lo = mid;
+      else hi = mid;
+    }
+    guide[j] = lo;
+  }
+}
+
+// CTA r: the conditional CDF of row r, its cutpoints, and the row's total into cdf_m[r + 1].
+__global__ void __launch_bounds__(kCdfThreads)
+env_cdf_rows_kernel(const float4* __restrict__ env, int W, float* __restrict__ cdf_m, float* __restrict__ cdf_c,
+                    int* __restrict__ guide_c, int gc_shift) {
+  extern __shared__ float4 cdf_smem4[];
+  float* v = reinterpret_cast<float*>(cdf_smem4);
+  const int r = blockIdx.x;
+  for (int c = threadIdx.x; c < W; c += kCdfThreads) {
     const float4 e = env[(size_t)r * W + c];
-    float lum = __fadd_rn(__fadd_rn(__fmul_rn(e.x, 0.2126f), __fmul_rn(e.y, 0.7152f)), __fmul_rn(e.z, 0.0722f));
-    lum = __fadd_rn(fmaxf(lum, 0.0f), 1e-6f);
-    s = __fadd_rn(s, lum);
-    row[c + 1] = s;
+    const float lum = __fadd_rn(__fadd_rn(__fmul_rn(e.x, 0.2126f), __fmul_rn(e.y, 0.7152f)), __fmul_rn(e.z, 0.0722f));
+    v[c] = __fadd_rn(fmaxf(lum, 0.0f), 1e-6f);
   }
-  for (int c = 1; c < W; ++c) row[c] = __fdiv_rn(row[c], s);
-  row[W] = 1.0f;
-  cdf_m[r + 1] = s;   // the row total, turned into the marginal CDF below
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    running_sum(v, W);
+    cdf_m[r + 1] = v[W - 1];   // turned into the marginal CDF below
+  }
+  __syncthreads();
+  finish_cdf(v, W, cdf_c + (size_t)r * (W + 1), guide_c + ((size_t)r << gc_shift), gc_shift);
 }
 
-__global__ void env_cdf_marginal_kernel(int H, float* __restrict__ cdf_m) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
-  cdf_m[0] = 0.0f;
-  float s = 0.0f;
-  for (int r = 1; r <= H; ++r) {
-    s = __fadd_rn(s, cdf_m[r]);
-    cdf_m[r] = s;
-  }
-  for (int r = 1; r < H; ++r) cdf_m[r] = __fdiv_rn(cdf_m[r], s);
-  cdf_m[H] = 1.0f;
-}
-
-// Cutpoint tables: entry j of a CDF's table is the bisection's answer for
-// u = j / 2^shift (exact in float32); thread per entry, the marginal's
-// table in row -1.
-__global__ void env_guide_kernel(int H, int W, const float* __restrict__ cdf_m, const float* __restrict__ cdf_c,
-                                 int* __restrict__ guide_m, int gm_shift, int* __restrict__ guide_c, int gc_shift) {
-  const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long Gm = 1LL << gm_shift, Gc = 1LL << gc_shift;
-  if (k < Gm) {
-    guide_m[k] = cdf_find(cdf_m, H, (float)k * (1.0f / (float)Gm));
-    return;
-  }
-  const long long e = k - Gm;
-  if (e >= (long long)H * Gc) return;
-  const long long r = e >> gc_shift, j = e & (Gc - 1);
-  guide_c[e] = cdf_find(cdf_c + r * (W + 1), W, (float)j * (1.0f / (float)Gc));
+// One CTA: the marginal CDF of the row totals in cdf_m[1..H], in place, and its cutpoints.
+__global__ void __launch_bounds__(kCdfThreads)
+env_cdf_marginal_kernel(int H, float* __restrict__ cdf_m, int* __restrict__ guide_m, int gm_shift) {
+  extern __shared__ float4 cdf_smem4[];
+  float* v = reinterpret_cast<float*>(cdf_smem4);
+  for (int r = threadIdx.x; r < H; r += kCdfThreads) v[r] = cdf_m[r + 1];
+  __syncthreads();
+  if (threadIdx.x == 0) running_sum(v, H);
+  __syncthreads();
+  finish_cdf(v, H, cdf_m, guide_m, gm_shift);
 }
 
 }  // namespace
 
 cudaError_t launch_env_cdf(const float4* env, int H, int W, float* cdf_m, float* cdf_c, int* guide_m, int gm_shift,
                            int* guide_c, int gc_shift, cudaStream_t s) {
-  env_cdf_rows_kernel<<<(H + 127) / 128, 128, 0, s>>>(env, H, W, cdf_m, cdf_c);
+  // a row of at most 8192 floats fits the 48 KB of shared memory that need no opt-in
+  env_cdf_rows_kernel<<<H, kCdfThreads, ((size_t)W + 3) / 4 * 16, s>>>(env, W, cdf_m, cdf_c, guide_c, gc_shift);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  env_cdf_marginal_kernel<<<1, 32, 0, s>>>(H, cdf_m);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  const long long n = (1LL << gm_shift) + (long long)H * (1LL << gc_shift);
-  env_guide_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(H, W, cdf_m, cdf_c, guide_m, gm_shift, guide_c,
-                                                               gc_shift);
+  env_cdf_marginal_kernel<<<1, kCdfThreads, ((size_t)H + 3) / 4 * 16, s>>>(H, cdf_m, guide_m, gm_shift);
   return cudaGetLastError();
 }
 

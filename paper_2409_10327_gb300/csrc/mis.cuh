@@ -19,21 +19,11 @@ namespace rtk {
 
 constexpr float kMisNovMin = 1e-4f;
 
-// largest k in [0, n - 1] with cdf[k] <= u, for cdf[0] = 0 <= u < cdf[n] = 1
-__device__ __forceinline__ int cdf_find(const float* __restrict__ cdf, int n, float u) {
-  int lo = 0, hi = n;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (__ldg(cdf + mid) <= u) lo = mid;
-    else hi = mid;
-  }
-  return lo;
-}
-
-// cdf_find with a cutpoint table (Chen & Asau's guide table): guide[j] =
-// cdf_find(cdf, n, j / G) for G = 2^gshift.  For u in [j, j + 1) / G the
-// answer lies in [guide[j], guide[j + 1]] because the CDF does not decrease,
-// so the bisection over that range returns the same index as over [0, n).
+// Largest k in [0, n - 1] with cdf[k] <= u, for cdf[0] = 0 <= u < cdf[n] = 1,
+// by a cutpoint table (Chen & Asau's guide table): guide[j] is that index for
+// u = j / G, G = 2^gshift.  For u in [j, j + 1) / G the answer lies in
+// [guide[j], guide[j + 1]] because the CDF does not decrease, so the bisection
+// over that range returns the same index as over [0, n).
 __device__ __forceinline__ int cdf_find_guided(const float* __restrict__ cdf, int n, float u,
                                                const int* __restrict__ guide, int gshift) {
   const int G = 1 << gshift;
