@@ -365,7 +365,7 @@ rt_status rt_decode(rt_ctx* ctx, const float* feat, int64_t P, float* brdf, void
   if (P < 0 || P > kMaxP) return RT_ERR_INVALID_ARG;
   if (P == 0) return RT_OK;
   if (feat == nullptr || !aligned(feat, 4) || brdf == nullptr || !aligned(brdf, 16)) return RT_ERR_INVALID_ARG;
-  return cuda_status(launch_decode(model_desc(ctx), feat, (int)P, brdf, (cudaStream_t)stream));
+  return cuda_status(launch_decode(model_desc(ctx), feat, (int)P, brdf, ctx->num_sms, (cudaStream_t)stream));
 }
 
 rt_status rt_trace(rt_ctx* ctx, const float* feat, const float* dirs, int64_t P, int32_t K, float* vis,

@@ -124,7 +124,7 @@ cudaError_t prepare_kernels();
 cudaError_t launch_repack(const float* brdf_w, const float* irt_w, int lf, float* wpack, cudaStream_t s);
 cudaError_t launch_encode(const ModelDesc& m, const float4* pos, int P, float* feat, uint32_t* idx,
                           float* w, cudaStream_t s);
-cudaError_t launch_decode(const ModelDesc& m, const float* feat, int P, float* brdf, cudaStream_t s);
+cudaError_t launch_decode(const ModelDesc& m, const float* feat, int P, float* brdf, int num_sms, cudaStream_t s);
 cudaError_t launch_trace(const ModelDesc& m, const float* feat, const float4* dirs, int P, int K,
                          float* vis, float* depth, int num_sms, cudaStream_t s);
 cudaError_t launch_sample(const ModelDesc& m, const float4* normal, int P, int level, long long offset,

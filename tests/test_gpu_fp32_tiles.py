@@ -1,0 +1,49 @@
+"""The FP32 kernels where their tiles can go wrong: rows that fill no tile, tiles of many points.
+
+Tolerances are those the same quantities have elsewhere (test_gpu_stages); the sizes put the edges of the 128-row tiles
+and of the per-point slots inside the data.
+"""
+import numpy as np
+import pytest
+import torch
+
+import scenegen
+from oracle import mlp
+from tests import helpers
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lib():
+    from paper_2409_10327_gb300 import build
+    build.build()
+    from paper_2409_10327_gb300 import binding
+    return binding
+
+
+# rows = 1, 127, 128, 129 and one tile over the number of warpgroups; K = 1 and 3: more points in a tile than slots
+@pytest.mark.parametrize("P, K", [(1, 1), (127, 1), (43, 3), (32, 4), (129, 1), (7, 17), (2600, 15)])
+def test_mlp_rows(lib, P, K):
+    cfg = helpers.small_cfg(levels=5)
+    sc = scenegen.make_scene(cfg, 6, bias_scale=0.3)
+    r = helpers.renderer_for(cfg, sc)
+    rng = np.random.default_rng(P + K)
+    feat = rng.normal(0, 0.2, (P, 10)).astype(np.float32)
+    d = rng.normal(size=(P, K, 3))
+    d /= np.linalg.norm(d, axis=-1, keepdims=True)
+    dirs = np.zeros((P, K, 4), np.float32)
+    dirs[..., :3] = d
+    f = torch.from_numpy(feat).cuda()
+    vis, depth = r.trace(f, torch.from_numpy(dirs).cuda())
+    out = r.decode(f).cpu().numpy()
+    f64 = torch.from_numpy(np.repeat(feat.astype(np.float64), K, axis=0))
+    v_ref, t_ref = mlp.implicit_ray_tracer(f64, torch.from_numpy(dirs[..., :3].reshape(-1, 3).astype(np.float64)),
+                                           mlp.as_layers(sc.irt), cfg.near, cfg.far)
+    np.testing.assert_allclose(vis.cpu().numpy().ravel(), v_ref.numpy(), atol=3e-6)
+    np.testing.assert_allclose(depth.cpu().numpy().ravel(), t_ref.numpy(), atol=3e-6)
+    a, rr, n = mlp.brdf_decoder(torch.from_numpy(feat.astype(np.float64)), mlp.as_layers(sc.brdf))
+    np.testing.assert_allclose(out[:, 0:3], n.numpy(), atol=2e-6)
+    np.testing.assert_allclose(out[:, 3:6], a.numpy(), atol=2e-6)
+    np.testing.assert_allclose(out[:, 6], rr.numpy(), atol=2e-6)
+    assert np.all(out[:, 7] == 0) and r.check() == 0
