@@ -1,22 +1,49 @@
 // Shared pieces of the hand-written FP32 adjoints (rt_backward, rt_distill_backward):
-// the per-CTA weight-gradient accumulator of I in shared memory (I runs 1 + M
-// times per row chunk; B, which runs once, adds its gradients straight into
-// the caller's blob with global atomics: BlobB gives its offsets), the warp-level
-// adjoints of the MLP layers (one row per lane, activations in the k-major
-// layout of warp_gemm.cuh) and of the trilinear hash encode, and the flush
-// of the accumulator into the caller's gradient blobs.
+// the warp-level adjoints of the MLP layers (32 rows per warp, activations in
+// the k-major layout of warp_gemm.cuh), the accumulators of I's weight
+// gradients, the adjoint of the trilinear hash encode, and the flush of the
+// accumulators into the caller's gradient blob.
+//
+// I runs 1 + M times per row chunk (B once), so its layers are all register
+// tiles: the forward and the transposed products (dZ1 = dZ2 W2, against a
+// transposed copy of W2 in shared memory) are 32 x 64 warp GEMMs, and a weight
+// gradient is a 64 x 64 (64 x 32) outer product over the warp's 32 rows with
+// 64 outputs per lane.  Its sum over the whole launch lives in tensor memory,
+// used as 256 words of private storage per lane (8 warps, two per TMEM lane
+// quarter): a chunk's 64 x 64 contribution is summed in registers and added
+// to the warp's accumulator by one tcgen05.ld / st of the lane's 64 words.
+// (A shared-memory accumulator per CTA took 246 float atomics per lane and
+// evaluation, more time than the products.)  B adds its gradients straight
+// into the caller's blob with coalesced global reductions (BlobB).
+// Bound by FMA chains and their shared-memory reads at two warps per
+// scheduler.  16,384 rays x 64 directions: 13.7 ms, about 30 ms with the
+// thread-per-row products and shared atomics; the distillation's kernel on
+// 2,048 points x 1,024 directions 1.53 ms, 4.5 ms before.
 #pragma once
 
+#include "tc_common.cuh"
 #include "warp_gemm.cuh"
 
 namespace rtk {
 
-// I's gradient accumulator in shared memory (floats; rows padded to K + 1)
-constexpr int LD_I1 = 60;                  // >= L*F + 27 + 1
-constexpr int LD_2 = 65;
-constexpr int GI_W1 = 0, GI_B1 = GI_W1 + 64 * LD_I1, GI_W2 = GI_B1 + 64, GI_B2 = GI_W2 + 64 * LD_2;
-constexpr int GI_W3 = GI_B2 + 64, GI_B3 = GI_W3 + 2 * LD_2;
-constexpr int G_FLOATS = (GI_B3 + 2 + 3) / 4 * 4;
+// Shared-memory weights of an adjoint: I's part of the packed image, then W2 transposed, [out c][in k]
+constexpr int OFF_IW2T = OFF_BW1;
+constexpr int WADJ_FLOATS = OFF_IW2T + 64 * 64;
+static_assert(OFF_IW2T % 4 == 0, "float4 alignment");
+
+constexpr int kAdjWarps = 8;               // warps per CTA, one CTA per SM
+constexpr int kAdjThreads = 32 * kAdjWarps;
+// TMEM words of a lane
+constexpr int TA_W2 = 0;                   // dW2, two passes of 64
+constexpr int TA_W1P = 128;                // dW1, PE columns
+constexpr int TA_S = 192;                  // backward: the chunk's sum over j of dZ1
+
+__device__ __forceinline__ void load_adjoint_weights(float* sw, const float* __restrict__ wpack) {
+  for (int i = threadIdx.x; i < OFF_BW1 / 4; i += kAdjThreads)
+    reinterpret_cast<float4*>(sw)[i] = __ldg(reinterpret_cast<const float4*>(wpack) + i);
+  for (int i = threadIdx.x; i < 4096; i += kAdjThreads)
+    sw[OFF_IW2T + i] = __ldg(wpack + OFF_IW2 + (i & 63) * 64 + (i >> 6));
+}
 
 // B's gradient blob (canonical layout of rt_param_count: W1 [64][lf], b1, W2 [64][64], b2, W3 [7][64], b3)
 struct BlobB {
@@ -29,6 +56,238 @@ struct BlobB {
   __device__ __forceinline__ float* w3() const { return g + 64 * lf + 128 + 4096; }
   __device__ __forceinline__ float* b3() const { return g + 64 * lf + 128 + 4096 + 448; }
 };
+
+// ---- tensor memory as per-lane accumulators --------------------------------
+__device__ __forceinline__ uint32_t adj_tmem_alloc(uint32_t* slot, int tid) {
+  if (tid < 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(slot)),
+                 "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  // warp w owns its 32 lanes (w % 4) and columns 256 (w / 4) ..
+  return *slot + ((uint32_t)(32 * ((tid >> 5) & 3)) << 16) + (uint32_t)(256 * (tid >> 7));
+}
+// called by all threads after their last TMEM access
+__device__ __forceinline__ void adj_tmem_free(const uint32_t* slot, int tid) {
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (tid < 32)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*slot), "r"(512) : "memory");
+}
+// words [0, 16 * n16) of this lane <- 0
+__device__ __forceinline__ void tmem_zero(uint32_t taddr, int n16) {
+  uint32_t z[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) z[i] = 0u;
+  for (int i = 0; i < n16; ++i) tmem_st16(taddr + 16 * i, z);
+  tmem_st_wait();
+}
+// 64 words of this lane += v
+__device__ __forceinline__ void tmem_add64(uint32_t taddr, const float (&v)[64]) {
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    uint32_t r[16];
+    tmem_ld16(taddr + 16 * h, r);
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) + v[16 * h + i]);
+    tmem_st16(taddr + 16 * h, r);
+  }
+  tmem_st_wait();
+}
+// the same for a Tile (words in v[q][c].x, .y order)
+__device__ __forceinline__ void tmem_add_tile(uint32_t taddr, const Tile& t) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    uint32_t r[16];
+    tmem_ld16(taddr + 16 * q, r);
+    tmem_ld_wait();
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      r[2 * c] = __float_as_uint(__uint_as_float(r[2 * c]) + t.v[q][c].x);
+      r[2 * c + 1] = __float_as_uint(__uint_as_float(r[2 * c + 1]) + t.v[q][c].y);
+    }
+    tmem_st16(taddr + 16 * q, r);
+  }
+  tmem_st_wait();
+}
+__device__ __forceinline__ void tmem_load_tile(uint32_t taddr, Tile& t) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    uint32_t r[16];
+    tmem_ld16(taddr + 16 * q, r);
+    tmem_ld_wait();
+#pragma unroll
+    for (int c = 0; c < 8; ++c) t.v[q][c] = make_float2(__uint_as_float(r[2 * c]), __uint_as_float(r[2 * c + 1]));
+  }
+}
+
+// ---- I's layers -------------------------------------------------------------
+// Columns (hidden units) of a lane where it owns two whole columns: the 8 lanes
+// of a quarter warp differ in c >> 3, so their float4 row reads hit distinct banks.
+__device__ __forceinline__ int own_col(int lane, int kk) { return 8 * (lane & 7) + (lane >> 3) + 4 * kk; }
+
+// Output layer: dZ2(c, row) = (sum_o dz[o][row] W3[c][o]) * [H2(c, row) > 0] over H2 in place, and for the lane's
+// two columns gw[kk][o] += sum_rows H2 dz[o], gb[kk] += sum_rows dZ2.  W3 is [64][2].
+template <int NOUT>
+__device__ __forceinline__ void bwd_out(float* H2, const float* dz, const float* W3, float (&gw)[2][2], float (&gb)[2],
+                                        int lane) {
+#pragma unroll
+  for (int kk = 0; kk < 2; ++kk) {
+    const int c = own_col(lane, kk);
+    const float w0 = W3[2 * c], w1 = NOUT > 1 ? W3[2 * c + 1] : 0.0f;
+    float s0 = 0.f, s1 = 0.f, sb = 0.f;
+#pragma unroll
+    for (int r = 0; r < 32; r += 4) {
+      float4* hp = reinterpret_cast<float4*>(H2 + aidx(c, r));
+      const float4 h4 = *hp, z4 = *reinterpret_cast<const float4*>(dz + r);
+      const float4 y4 = NOUT > 1 ? *reinterpret_cast<const float4*>(dz + 32 + r) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float h[4] = {h4.x, h4.y, h4.z, h4.w}, z[4] = {z4.x, z4.y, z4.z, z4.w}, y[4] = {y4.x, y4.y, y4.z, y4.w};
+      float g[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        g[u] = z[u] * w0;
+        if (NOUT > 1) g[u] = fmaf(y[u], w1, g[u]);
+        g[u] = h[u] > 0.0f ? g[u] : 0.0f;
+        sb += g[u];
+        s0 = fmaf(h[u], z[u], s0);
+        if (NOUT > 1) s1 = fmaf(h[u], y[u], s1);
+      }
+      *hp = make_float4(g[0], g[1], g[2], g[3]);
+    }
+    gw[kk][0] += s0;
+    if (NOUT > 1) gw[kk][1] += s1;
+    gb[kk] += sb;
+  }
+}
+
+// One outer product over the warp's rows: v[i * NK + j] = sum_rows D(c0 + i, row) A(k0 + j, row), 64 outputs a lane.
+template <int NC, int NK>
+__device__ __forceinline__ void outer64(const float* A, const float* D, int k0, int c0, float (&v)[64]) {
+  static_assert(NC * NK == 64, "64 outputs per lane");
+#pragma unroll
+  for (int i = 0; i < 64; ++i) v[i] = 0.0f;
+#pragma unroll 1
+  for (int r = 0; r < 32; r += 4) {
+    float4 a[NK];
+#pragma unroll
+    for (int j = 0; j < NK; ++j) a[j] = *reinterpret_cast<const float4*>(A + aidx(k0 + j, r));
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      const float4 d = *reinterpret_cast<const float4*>(D + aidx(c0 + i, r));
+#pragma unroll
+      for (int j = 0; j < NK; ++j) {
+        float s = v[i * NK + j];
+        s = fmaf(a[j].x, d.x, s);
+        s = fmaf(a[j].y, d.y, s);
+        s = fmaf(a[j].z, d.z, s);
+        v[i * NK + j] = fmaf(a[j].w, d.w, s);
+      }
+    }
+  }
+}
+// dW2 += dZ2^T H1 into the warp's accumulator (lane: rows c = 32 pass + 8 rg.., columns k = 8 cg..)
+__device__ __forceinline__ void acc_w2(const float* H1, const float* DZ2, uint32_t tacc, int rg, int cg) {
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+    float v[64];
+    outer64<8, 8>(H1, DZ2, 8 * cg, 32 * pass + 8 * rg, v);
+    tmem_add64(tacc + TA_W2 + 64 * pass, v);
+  }
+}
+// dW1's PE columns += dZ1^T PE (lane: rows c = 16 rg.., columns k = 4 cg..)
+__device__ __forceinline__ void acc_w1p(const float* PE, const float* DZ1, uint32_t tacc, int rg, int cg) {
+  float v[64];
+  outer64<16, 4>(PE, DZ1, 4 * cg, 16 * rg, v);
+  tmem_add64(tacc + TA_W1P, v);
+}
+
+// dZ1 = (dZ2 W2) masked by H1 > 0, over H1 in place (t: the masked tile).  Every lane has read H1 before.
+__device__ __forceinline__ void bwd_hidden_tile(const float* DZ2, const float* W2T, float* H1, Tile& t, int rg, int cg) {
+  zero(t);
+  warp_gemm<kHidden>(DZ2, W2T, t, rg, cg);
+  __syncwarp();
+  store_masked(H1, t, rg, cg);
+  __syncwarp();
+}
+
+// sum over the warp's rows of the lane's two columns
+__device__ __forceinline__ void col_sums(const float* D, float (&s)[2], int lane) {
+#pragma unroll
+  for (int kk = 0; kk < 2; ++kk) {
+    float a = 0.0f;
+#pragma unroll
+    for (int r = 0; r < 32; r += 4) {
+      const float4 d = *reinterpret_cast<const float4*>(D + aidx(own_col(lane, kk), r));
+      a += (d.x + d.y) + (d.z + d.w);
+    }
+    s[kk] += a;
+  }
+}
+
+// Where f is shared by the rows (a pixel's or a point's directions), with cs[c] the sum over rows of dZ1:
+// dW1f[c][k] += f[k] cs[c] (coalesced global reductions) and, returned in lane k, dLoss/df[k] = sum_c cs[c] W1f[k][c].
+__device__ __forceinline__ float bwd_shared_feature(const float* f, const float* cs, const float* W1F, int lf,
+                                                    float* __restrict__ g_irt, int lane) {
+  float s = 0.0f;
+  if (lane < lf) {
+    const int in_i = lf + kPE;
+    const float fk = f[lane];
+#pragma unroll 8
+    for (int c = 0; c < 64; ++c) atomicAdd(g_irt + c * in_i + lane, fk * cs[c]);
+#pragma unroll 8
+    for (int cc = 0; cc < 64; ++cc) {
+      const int c = (cc + lane) & 63;   // rotated: the lanes' rows of W1F share banks
+      s = fmaf(cs[c], W1F[lane * 64 + c], s);
+    }
+  }
+  return s;
+}
+
+// gW[c][k] += sum_rows A(k, row) D(c, row) for c < 64, k < K, rows of gW ld apart: lane = k, so the reductions into
+// global memory are coalesced; gb[c] += sum_rows D(c, row) if gb != nullptr.
+__device__ __forceinline__ void bwd_weights_global(const float* A, int K, const float* D, float* __restrict__ gW, int ld,
+                                                   float* __restrict__ gb, int lane) {
+  for (int k0 = 0; k0 < K; k0 += 32) {
+    const int k = k0 + lane;
+    const bool live = k < K;
+    float a[32];
+#pragma unroll
+    for (int r = 0; r < 32; r += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(A + aidx(live ? k : k0, r));
+      a[r] = v.x;
+      a[r + 1] = v.y;
+      a[r + 2] = v.z;
+      a[r + 3] = v.w;
+    }
+    for (int c = 0; c < 64; ++c) {
+      float s = 0.0f;
+#pragma unroll
+      for (int r = 0; r < 32; r += 4) {
+        const float4 d = *reinterpret_cast<const float4*>(D + aidx(c, r));
+        s = fmaf(a[r], d.x, s);
+        s = fmaf(a[r + 1], d.y, s);
+        s = fmaf(a[r + 2], d.z, s);
+        s = fmaf(a[r + 3], d.w, s);
+      }
+      if (live) atomicAdd(gW + c * ld + k, s);
+    }
+  }
+  if (gb != nullptr) {
+    float s[2] = {0.f, 0.f};
+    col_sums(D, s, lane);
+    atomicAdd(gb + own_col(lane, 0), s[0]);
+    atomicAdd(gb + own_col(lane, 1), s[1]);
+  }
+}
+
+// ---- B's layers (one evaluation per chunk; weights through the read-only cache) ----
 // DZ2(c, row) = (sum_o dz[o][row] W3[c][o]) * [H2(c, row) > 0]   (thread per row)
 template <int NOUT, int LDW>
 __device__ __forceinline__ void bwd_head(const float* H2, const float* dz, const float* W3, float* DZ2, int lane) {
@@ -39,25 +298,27 @@ __device__ __forceinline__ void bwd_head(const float* H2, const float* dz, const
   for (int c = 0; c < 64; ++c) {
     float s = 0.0f;
 #pragma unroll
-    for (int o = 0; o < NOUT; ++o) s = fmaf(g[o], W3[c * LDW + o], s);
+    for (int o = 0; o < NOUT; ++o) s = fmaf(g[o], __ldg(W3 + c * LDW + o), s);
     DZ2[aidx(c, lane)] = H2[aidx(c, lane)] > 0.0f ? s : 0.0f;
   }
 }
 
 // dW3[o][k] += sum_rows H2(k, row) dz[o][row]; db3[o] += sum_rows dz[o][row]
 template <int NOUT>
-__device__ __forceinline__ void bwd_w3(const float* H2, const float* dz, float* gW3, float* gb3, int lane,
-                                       int ld = LD_2) {
+__device__ __forceinline__ void bwd_w3(const float* H2, const float* dz, float* gW3, float* gb3, int lane, int ld) {
 #pragma unroll 1   // rolled: unrolled, the two passes' global atomics keep too many registers live
   for (int kk = 0; kk < 2; ++kk) {
-    const int k = 2 * lane + kk;
+    const int k = own_col(lane, kk);
     float acc[NOUT];
 #pragma unroll
     for (int o = 0; o < NOUT; ++o) acc[o] = 0.0f;
-    for (int r = 0; r < 32; ++r) {
-      const float h = H2[aidx(k, r)];
+    for (int r = 0; r < 32; r += 4) {
+      const float4 h = *reinterpret_cast<const float4*>(H2 + aidx(k, r));
 #pragma unroll
-      for (int o = 0; o < NOUT; ++o) acc[o] = fmaf(h, dz[o * 32 + r], acc[o]);
+      for (int o = 0; o < NOUT; ++o) {
+        const float4 z = *reinterpret_cast<const float4*>(dz + o * 32 + r);
+        acc[o] = fmaf(h.w, z.w, fmaf(h.z, z.z, fmaf(h.y, z.y, fmaf(h.x, z.x, acc[o]))));
+      }
     }
 #pragma unroll
     for (int o = 0; o < NOUT; ++o) atomicAdd(gW3 + o * ld + k, acc[o]);
@@ -69,54 +330,19 @@ __device__ __forceinline__ void bwd_w3(const float* H2, const float* dz, float* 
   }
 }
 
-// dW[c][koff + k] += sum_rows A(k, row) D(c, row) for k < K, c in {2 lane, 2 lane + 1};
-// if gb != nullptr also db[c] += sum_rows D(c, row)
-__device__ __forceinline__ void bwd_weights(const float* A, int K, const float* D, float* gW, int ld, int koff,
-                                            float* gb, int lane) {
-#pragma unroll
-  for (int cc = 0; cc < 2; ++cc) {
-    const int c = 2 * lane + cc;
-    float d[32];
-#pragma unroll
-    for (int r = 0; r < 32; r += 4) {
-      const float4 v = *reinterpret_cast<const float4*>(D + aidx(c, r));
-      d[r] = v.x;
-      d[r + 1] = v.y;
-      d[r + 2] = v.z;
-      d[r + 3] = v.w;
-    }
-    if (gb != nullptr) {
-      float s = 0.0f;
-#pragma unroll
-      for (int r = 0; r < 32; ++r) s += d[r];
-      atomicAdd(gb + c, s);
-    }
-    for (int k = 0; k < K; ++k) {
-      float s = 0.0f;
-#pragma unroll
-      for (int r = 0; r < 32; r += 4) {
-        const float4 a = *reinterpret_cast<const float4*>(A + aidx(k, r));
-        s = fmaf(a.x, d[r], s);
-        s = fmaf(a.y, d[r + 1], s);
-        s = fmaf(a.z, d[r + 2], s);
-        s = fmaf(a.w, d[r + 3], s);
-      }
-      atomicAdd(gW + c * ld + koff + k, s);
-    }
-  }
-}
-
 // OUT(k, row) = (sum_c D(c, row) W[k][c]) * [MASK(k, row) > 0] for k < 64 (thread per row);
-// W is a [64][64] shared matrix stored [k][c]
-__device__ __forceinline__ void bwd_hidden(const float* D, const float* W, const float* MASK, float* OUT, int lane) {
+// W is a [64][64] matrix in global memory stored [k][c]
+__device__ __forceinline__ void bwd_hidden(const float* D, const float* __restrict__ W, const float* MASK, float* OUT,
+                                           int lane) {
   float d[64];
 #pragma unroll
   for (int c = 0; c < 64; ++c) d[c] = D[aidx(c, lane)];
+#pragma unroll 2
   for (int k = 0; k < 64; ++k) {
     float s = 0.0f;
 #pragma unroll
     for (int c = 0; c < 64; c += 4) {
-      const float4 w = *reinterpret_cast<const float4*>(W + k * 64 + c);
+      const float4 w = __ldg(reinterpret_cast<const float4*>(W + k * 64 + c));
       s = fmaf(d[c], w.x, s);
       s = fmaf(d[c + 1], w.y, s);
       s = fmaf(d[c + 2], w.z, s);
@@ -365,19 +591,73 @@ __device__ __forceinline__ float spec_with_grad(float rough, f3 n, f3 wi, f3 wo,
   return D * F * vis;
 }
 
-// Add the CTA's accumulated gradients of I into the caller's blob (canonical
-// layout of rt_param_count); called by all threads after a barrier.
-__device__ __forceinline__ void flush_irt_grads(const float* sg, int lf, float* __restrict__ g_irt, int nthreads) {
+// ---- I's weight gradients to the caller -------------------------------------
+// The gradients a lane keeps in registers: for its two columns dW3, db2 and db1, and its rows' db3.
+struct IrtGrads {
+  float w3[2][2], b2[2], b1[2], b3[2];
+};
+__device__ __forceinline__ void zero(IrtGrads& g) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) g.w3[i][0] = g.w3[i][1] = g.b2[i] = g.b1[i] = g.b3[i] = 0.0f;
+}
+
+// Sum the warps' accumulators over the CTA in shared memory (buf: kAdjWarps blocks of 4160 floats, `stride` floats
+// apart) and add them to the caller's blob (canonical layout of rt_param_count), coalesced.  All threads call it.
+__device__ __forceinline__ void flush_irt_grads(float* buf, int stride, uint32_t tacc, IrtGrads& g, int lf,
+                                                float* __restrict__ g_irt) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rg = lane >> 3, cg = lane & 7;
   const int in_i = lf + kPE;
-  const int iW1 = 0, iB1 = 64 * in_i, iW2 = iB1 + 64, iB2 = iW2 + 4096, iW3 = iB2 + 64, iB3 = iW3 + 128;
-  for (int e = threadIdx.x; e < 64 * in_i; e += nthreads) atomicAdd(g_irt + iW1 + e, sg[GI_W1 + (e / in_i) * LD_I1 + e % in_i]);
-  for (int e = threadIdx.x; e < 64; e += nthreads) {
-    atomicAdd(g_irt + iB1 + e, sg[GI_B1 + e]);
-    atomicAdd(g_irt + iB2 + e, sg[GI_B2 + e]);
+  const int iB1 = 64 * in_i, iW2 = iB1 + 64, iB2 = iW2 + 4096, iW3 = iB2 + 64, iB3 = iW3 + 128;
+  float* mine = buf + warp * stride;
+  auto cta_sum = [&](int e) {
+    float s = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kAdjWarps; ++w) s += buf[w * stride + e];
+    return s;
+  };
+  __syncthreads();
+#pragma unroll 1
+  for (int part = 0; part < 3; ++part) {   // the two halves of dW2, then dW1's PE columns
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      uint32_t r[16];
+      tmem_ld16(tacc + 64 * part + 16 * h, r);
+      tmem_ld_wait();
+#pragma unroll
+      for (int i = 0; i < 16; i += 4) {
+        const int e = 16 * h + i;
+        // parts 0, 1: [32 rows][64]; part 2: [64 rows][32]
+        const int o = part < 2 ? (8 * rg + (e >> 3)) * 64 + 8 * cg + (e & 7) : (16 * rg + (e >> 2)) * 32 + 4 * cg;
+        *reinterpret_cast<float4*>(mine + o) = make_float4(__uint_as_float(r[i]), __uint_as_float(r[i + 1]),
+                                                           __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
+      }
+    }
+    __syncthreads();
+    for (int e = tid; e < 2048; e += kAdjThreads) {
+      if (part < 2) atomicAdd(g_irt + iW2 + 2048 * part + e, cta_sum(e));
+      else if ((e & 31) < kPE) atomicAdd(g_irt + (e >> 5) * in_i + lf + (e & 31), cta_sum(e));
+    }
+    __syncthreads();
   }
-  for (int e = threadIdx.x; e < 4096; e += nthreads) atomicAdd(g_irt + iW2 + e, sg[GI_W2 + (e / 64) * LD_2 + e % 64]);
-  for (int e = threadIdx.x; e < 128; e += nthreads) atomicAdd(g_irt + iW3 + e, sg[GI_W3 + (e / 64) * LD_2 + e % 64]);
-  for (int e = threadIdx.x; e < 2; e += nthreads) atomicAdd(g_irt + iB3 + e, sg[GI_B3 + e]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    g.b3[0] += __shfl_xor_sync(0xffffffffu, g.b3[0], o);
+    g.b3[1] += __shfl_xor_sync(0xffffffffu, g.b3[1], o);
+  }
+#pragma unroll
+  for (int kk = 0; kk < 2; ++kk) {
+    const int c = own_col(lane, kk);
+    mine[c] = g.w3[kk][0];
+    mine[64 + c] = g.w3[kk][1];
+    mine[128 + c] = g.b2[kk];
+    mine[192 + c] = g.b1[kk];
+  }
+  if (lane < 2) mine[256 + lane] = g.b3[lane];
+  __syncthreads();
+  for (int e = tid; e < 258; e += kAdjThreads) {
+    const int o = e < 128 ? iW3 + e : e < 192 ? iB2 + e - 128 : e < 256 ? iB1 + e - 192 : iB3 + e - 256;
+    atomicAdd(g_irt + o, cta_sum(e));
+  }
 }
 
 }  // namespace rtk

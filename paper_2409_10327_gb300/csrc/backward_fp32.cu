@@ -18,10 +18,11 @@
 //      dz0 from dv = dL_i . (Lenv(w_i) - L'_o,i), and back-propagates the
 //      primary I (recomputed) into its weights and into dLoss/df.
 // After the pixel's last chunk the primary encode scatters dLoss/df into the
-// table.  Weight gradients of each chunk are small warp GEMMs.  I's (1 + M
-// evaluations per chunk) are added to a per-CTA shared-memory accumulator
-// (padded rows, shared atomics) that the CTA adds to the caller's blob once at
-// the end; B's (one evaluation per chunk) go to the caller's blob directly.
+// table.  What a chunk's M evaluations share is done once per chunk: layer 1's
+// b1 + W1f f' enters as a register tile, and since f' is the same for all of
+// them the f' parts of dW1 and of dLoss/df' take the sum of dZ1 over j.
+// Weight gradients are 32-row outer products; adjoint.cuh says where each is
+// summed.
 // With MIS primary directions (Sec. 4.1) each draw and its weight are
 // constants too; only w_i and its Eq. 1 factor change.
 #include "adjoint.cuh"
@@ -31,42 +32,38 @@ namespace rtk {
 
 namespace {
 
-constexpr int kBW = 6;                     // warps per CTA
-constexpr int kBT = 32 * kBW;
 // per-warp buffers (floats)
 constexpr int WB_F2 = 0;                                   // f' of the chunk's rows  [32 cols]
 constexpr int WB_H1 = WB_F2 + kActStride32;                 // layer-1 activations, then dZ1 (in place) [64 cols]
 // PE of the current direction [32 cols] for layer 1, then layer-2 activations and dZ2 (in place)
 // [64 cols]; the PE is written again for the PE part of dW1 once dZ2 is consumed
 constexpr int WB_H2 = WB_H1 + kActStride;
-constexpr int WB_DZ = WB_H2 + kActStride;                  // output gradients [8][32]
-constexpr int WB_FP = WB_DZ + 8 * 32;                       // primary feature f [32]
+constexpr int WB_DZ = WB_H2 + kActStride;                  // output gradients [7][32]; column sums [64]
+constexpr int WB_FP = WB_DZ + 7 * 32;                       // primary feature f [32]
 constexpr int WB_AP = WB_FP + 32;                           // primary b1 + W1f f [64]
-constexpr int WB_DFP = WB_AP + 64;                          // dLoss/df of the pixel [32]
-constexpr int WB_FLOATS = WB_DFP + 32;
-constexpr size_t kBSmem = (size_t)(WPACK_FLOATS + G_FLOATS + kBW * WB_FLOATS) * sizeof(float);
-static_assert(LD_I1 >= 32 + 27 + 1, "gradient rows");
+constexpr int WB_FLOATS = WB_AP + 64;
+constexpr size_t kBSmem = (size_t)(WADJ_FLOATS + kAdjWarps * WB_FLOATS + 4) * sizeof(float);
 static_assert(kBSmem <= 232448, "one CTA per SM");
-static_assert(WB_F2 % 4 == 0 && WB_H1 % 4 == 0 && WB_H2 % 4 == 0 &&
-                  WB_DZ % 4 == 0 && WB_FLOATS % 4 == 0 && G_FLOATS % 4 == 0,
+static_assert(WB_F2 % 4 == 0 && WB_H1 % 4 == 0 && WB_H2 % 4 == 0 && WB_H2 == WB_H1 + kActStride &&
+                  WB_DZ % 4 == 0 && WB_FLOATS % 4 == 0,
               "float4 alignment");
 
-// ---- warp-level pieces of an MLP backward -----------------------------------
-
-__global__ void __launch_bounds__(kBT, 1)
+__global__ void __launch_bounds__(kAdjThreads, 1)
 backward_fp32_kernel(ModelDesc m, rt_gbuffer gb, int P, long long pixel_offset, const float4* __restrict__ dL,
                      float* __restrict__ g_table, float* __restrict__ g_brdf, float* __restrict__ g_irt) {
   extern __shared__ float4 smem4[];
   float* sw = reinterpret_cast<float*>(smem4);
-  float* sg = sw + WPACK_FLOATS;
-  for (int i = threadIdx.x; i < WPACK_FLOATS / 4; i += kBT)
-    smem4[i] = __ldg(reinterpret_cast<const float4*>(m.wpack) + i);
-  for (int i = threadIdx.x; i < G_FLOATS; i += kBT) sg[i] = 0.0f;
-  __syncthreads();
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(sw + WADJ_FLOATS + kAdjWarps * WB_FLOATS);
+  load_adjoint_weights(sw, m.wpack);
+  const uint32_t tacc = adj_tmem_alloc(tslot, threadIdx.x);   // (its barrier also publishes the weights)
+  tmem_zero(tacc, 16);
+  IrtGrads gI;
+  zero(gI);
+  const float* bw = m.wpack;   // B's weights stay in global memory: one evaluation in nine or ten
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rg = lane >> 3, cg = lane & 7;
-  float* wb = sg + G_FLOATS + warp * WB_FLOATS;
+  float* wb = sw + WADJ_FLOATS + warp * WB_FLOATS;
   float* F2 = wb + WB_F2;
   float* PEb = wb + WB_H2;   // shares H2's buffer (see WB_H2)
   float* H1 = wb + WB_H1;
@@ -74,7 +71,6 @@ backward_fp32_kernel(ModelDesc m, rt_gbuffer gb, int P, long long pixel_offset, 
   float* DZ = wb + WB_DZ;
   float* fP = wb + WB_FP;
   float* aP = wb + WB_AP;
-  float* dfP = wb + WB_DFP;
   const int N = m.N, M = m.M, lf = m.lf, lfp = m.lfp;
   const bool disney = !m.lambert;
   const BlobB gB{g_brdf, lf};
@@ -83,7 +79,7 @@ backward_fp32_kernel(ModelDesc m, rt_gbuffer gb, int P, long long pixel_offset, 
   const float4* view4 = reinterpret_cast<const float4*>(gb.view);
   const float4* ar4 = reinterpret_cast<const float4*>(gb.albedo_rough);
 
-  for (int pix = blockIdx.x * kBW + warp; pix < P; pix += gridDim.x * kBW) {
+  for (int pix = blockIdx.x * kAdjWarps + warp; pix < P; pix += gridDim.x * kAdjWarps) {
     const f3 x = xyz(pos4[pix]);
     const f3 n = xyz(nrm4[pix]);
     const f3 wo = xyz(view4[pix]);
@@ -102,7 +98,6 @@ backward_fp32_kernel(ModelDesc m, rt_gbuffer gb, int P, long long pixel_offset, 
         fP[lane] = part.x;
         fP[lane + 1] = part.y;
       }
-      dfP[lane] = 0.0f;
     }
     __syncwarp();
 #pragma unroll
@@ -113,6 +108,7 @@ backward_fp32_kernel(ModelDesc m, rt_gbuffer gb, int P, long long pixel_offset, 
       aP[c] = acc;
     }
     __syncwarp();
+    float cs[2] = {0.f, 0.f};   // the pixel's sum of the primary evaluations' dZ1, the lane's two columns
 
     for (int i0 = 0; i0 < N; i0 += 32) {
       const int i = i0 + lane;
@@ -121,13 +117,13 @@ backward_fp32_kernel(ModelDesc m, rt_gbuffer gb, int P, long long pixel_offset, 
       // the primary direction and its Eq. 1 factor are constants of the estimator (MIS included)
       const f3 wi = m.mis ? mis_direction(m, n, wo, ar.w, i, dir_counter(q, M, 0))
                           : cosine_direction(n, m.seed, dir_counter(q, M, 0));
-      float acc[8][8];
+      Tile acc;
 
       // ---- forward of I(f, w_i)
       store_pe(PEb, wi, lane);
       __syncwarp();
       zero(acc);
-      warp_gemm<kPEPad>(PEb, sw + OFF_IW1P, acc, rg, cg);
+      warp_gemm<kPEPad - 4>(PEb, sw + OFF_IW1P, acc, rg, cg);
       store_relu_colbias(H1, acc, aP, rg, cg);
       __syncwarp();
       zero(acc);
@@ -150,20 +146,24 @@ backward_fp32_kernel(ModelDesc m, rt_gbuffer gb, int P, long long pixel_offset, 
       for (int k = lf; k < 32; ++k) F2[aidx(k, lane)] = 0.0f;
       __syncwarp();
       zero(acc);
-      warp_gemm_k(F2, sw + OFF_BW1, acc, lfp, rg, cg);
-      store_relu_colbias(H1, acc, sw + OFF_BB1, rg, cg);
+      warp_gemm_k(F2, bw + OFF_BW1, acc, lfp, rg, cg);
+      store_relu_colbias(H1, acc, bw + OFF_BB1, rg, cg);
       __syncwarp();
       zero(acc);
-      warp_gemm<kHidden>(H1, sw + OFF_BW2, acc, rg, cg);
-      store_relu_colbias(H2, acc, sw + OFF_BB2, rg, cg);
+      warp_gemm<kHidden>(H1, bw + OFF_BW2, acc, rg, cg);
+      store_relu_colbias(H2, acc, bw + OFF_BB2, rg, cg);
       __syncwarp();
       float y[7];
 #pragma unroll
-      for (int o = 0; o < 7; ++o) y[o] = sw[OFF_BB3 + o];
+      for (int o = 0; o < 7; ++o) y[o] = __ldg(bw + OFF_BB3 + o);
+#pragma unroll 4
       for (int k = 0; k < kHidden; ++k) {
         const float hk = H2[aidx(k, lane)];
+        const float4 w0 = __ldg(reinterpret_cast<const float4*>(bw + OFF_BW3 + 8 * k));
+        const float4 w1 = __ldg(reinterpret_cast<const float4*>(bw + OFF_BW3 + 8 * k + 4));
+        const float w[7] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z};
 #pragma unroll
-        for (int o = 0; o < 7; ++o) y[o] = fmaf(hk, sw[OFF_BW3 + 8 * k + o], y[o]);
+        for (int o = 0; o < 7; ++o) y[o] = fmaf(hk, w[o], y[o]);
       }
       const float nlen = sqrtf(fmaxf(y[0] * y[0] + y[1] * y[1] + y[2] * y[2], 1e-24f));
       const f3 n2 = mk(y[0] / nlen, y[1] / nlen, y[2] / nlen);
@@ -181,9 +181,15 @@ backward_fp32_kernel(ModelDesc m, rt_gbuffer gb, int P, long long pixel_offset, 
       const f3 dlo2 = dli * (1.0f - v);
 
       // ---- secondary directions: forward and backward of I(f', w'_j)
-      float dF2[32];
+      Tile a2b;   // I's layer-1 bias for the secondary point, b1 + W1f f'
+      zero(a2b);
+      warp_gemm_k(F2, sw + OFF_IW1F, a2b, lfp, rg, cg);
 #pragma unroll
-      for (int k = 0; k < 32; ++k) dF2[k] = 0.0f;
+      for (int c = 0; c < 8; ++c) {
+        const float b = sw[OFF_IB1 + ocol(cg, c)];
+#pragma unroll
+        for (int qq = 0; qq < 4; ++qq) a2b.v[qq][c] = make_float2(a2b.v[qq][c].x + b, a2b.v[qq][c].y + b);
+      }
       f3 lo2 = mk(0.f, 0.f, 0.f), da2 = mk(0.f, 0.f, 0.f), dn2 = mk(0.f, 0.f, 0.f);
       float dr2 = 0.0f;
       for (int j = 0; j < M; ++j) {
@@ -192,9 +198,8 @@ backward_fp32_kernel(ModelDesc m, rt_gbuffer gb, int P, long long pixel_offset, 
         store_pe(PEb, wj, lane);
         __syncwarp();
         zero(acc);
-        warp_gemm_k(F2, sw + OFF_IW1F, acc, lfp, rg, cg);
-        warp_gemm<kPEPad>(PEb, sw + OFF_IW1P, acc, rg, cg);
-        store_relu_colbias(H1, acc, sw + OFF_IB1, rg, cg);
+        warp_gemm<kPEPad - 4>(PEb, sw + OFF_IW1P, acc, rg, cg);
+        store_relu_tilebias(H1, acc, a2b, rg, cg);
         __syncwarp();
         zero(acc);
         warp_gemm<kHidden>(H1, sw + OFF_IW2, acc, rg, cg);
@@ -221,21 +226,35 @@ backward_fp32_kernel(ModelDesc m, rt_gbuffer gb, int P, long long pixel_offset, 
         const float dz0 = m.force_vis2 >= 0.f ? 0.0f : dv2 * v2 * (1.0f - v2);
         DZ[lane] = dz0;
         __syncwarp();
-        // I backward: head, W3, W2, hidden, W1 (f' and PE parts), input f'
-        bwd_w3<1>(H2, DZ, sg + GI_W3, sg + GI_B3, lane);
+        // I backward: output layer, W2, hidden, the PE part of W1; the sum of dZ1 over j for the f' part
+        gI.b3[0] += dz0;
+        bwd_out<1>(H2, DZ, sw + OFF_IW3, gI.w3, gI.b2, lane);
         __syncwarp();
-        bwd_head<1, 2>(H2, DZ, sw + OFF_IW3, H2, lane);   // dZ2 over H2, in place
+        acc_w2(H1, H2, tacc, rg, cg);
+        bwd_hidden_tile(H2, sw + OFF_IW2T, H1, acc, rg, cg);
+        tmem_add_tile(tacc + TA_S, acc);
+        store_pe(PEb, wj, lane);   // again, over the consumed dZ2
         __syncwarp();
-        bwd_weights(H1, 64, H2, sg + GI_W2, LD_2, 0, sg + GI_B2, lane);
-        __syncwarp();
-        bwd_hidden(H2, sw + OFF_IW2, H1, H1, lane);   // dZ1 over H1, in place
-        __syncwarp();
-        store_pe(PEb, cosine_direction(n2, m.seed, dir_counter(q, M, 1 + j)), lane);   // again, over dZ2
-        bwd_weights(F2, lf, H1, sg + GI_W1, LD_I1, 0, sg + GI_B1, lane);
-        __syncwarp();
-        bwd_weights(PEb, kPE, H1, sg + GI_W1, LD_I1, lf, nullptr, lane);
-        bwd_input(H1, sw + OFF_IW1F, lf, dF2, lane);
+        acc_w1p(PEb, H1, tacc, rg, cg);
       }
+      // the f' part of I's layer 1, and dLoss/df' of the secondary evaluations
+      float dF2[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) dF2[k] = 0.0f;
+      tmem_load_tile(tacc + TA_S, acc);
+      tmem_zero(tacc + TA_S, 4);
+      __syncwarp();
+      store_tile(H1, acc, rg, cg);
+      __syncwarp();
+      {
+        float s[2] = {0.f, 0.f};
+        col_sums(H1, s, lane);
+        gI.b1[0] += s[0];
+        gI.b1[1] += s[1];
+      }
+      bwd_weights_global(F2, lf, H1, g_irt, lf + kPE, nullptr, lane);
+      bwd_input(H1, sw + OFF_IW1F, lf, dF2, lane);
+      __syncwarp();
       lo2 = lo2 * sM;
       const float dv = dot(dli, e1 - lo2);
 
@@ -253,25 +272,25 @@ backward_fp32_kernel(ModelDesc m, rt_gbuffer gb, int P, long long pixel_offset, 
       }
       __syncwarp();
       zero(acc);
-      warp_gemm_k(F2, sw + OFF_BW1, acc, lfp, rg, cg);
-      store_relu_colbias(H1, acc, sw + OFF_BB1, rg, cg);
+      warp_gemm_k(F2, bw + OFF_BW1, acc, lfp, rg, cg);
+      store_relu_colbias(H1, acc, bw + OFF_BB1, rg, cg);
       __syncwarp();
       zero(acc);
-      warp_gemm<kHidden>(H1, sw + OFF_BW2, acc, rg, cg);
-      store_relu_colbias(H2, acc, sw + OFF_BB2, rg, cg);
+      warp_gemm<kHidden>(H1, bw + OFF_BW2, acc, rg, cg);
+      store_relu_colbias(H2, acc, bw + OFF_BB2, rg, cg);
 #pragma unroll
       for (int o = 0; o < 7; ++o) DZ[o * 32 + lane] = dy[o];
       __syncwarp();
       bwd_w3<7>(H2, DZ, gB.w3(), gB.b3(), lane, 64);
       __syncwarp();
-      bwd_head<7, 8>(H2, DZ, sw + OFF_BW3, H2, lane);   // dZ2 over H2, in place
+      bwd_head<7, 8>(H2, DZ, bw + OFF_BW3, H2, lane);   // dZ2 over H2, in place
       __syncwarp();
-      bwd_weights(H1, 64, H2, gB.w2(), 64, 0, gB.b2(), lane);
+      bwd_weights_global(H1, 64, H2, gB.w2(), 64, gB.b2(), lane);
       __syncwarp();
-      bwd_hidden(H2, sw + OFF_BW2, H1, H1, lane);   // dZ1 over H1, in place
+      bwd_hidden(H2, bw + OFF_BW2, H1, H1, lane);   // dZ1 over H1, in place
       __syncwarp();
-      bwd_weights(F2, lf, H1, gB.w1(), lf, 0, gB.b1(), lane);
-      bwd_input(H1, sw + OFF_BW1, lf, dF2, lane);
+      bwd_weights_global(F2, lf, H1, gB.w1(), lf, gB.b1(), lane);
+      bwd_input(H1, bw + OFF_BW1, lf, dF2, lane);
 
       // ---- encode adjoint at x': table gradients (segmented scatter over the warp's points in Morton
       // order) and dLoss/dx'; H2's buffer, free until the next store_pe, carries dx' back to its lane
@@ -288,62 +307,48 @@ backward_fp32_kernel(ModelDesc m, rt_gbuffer gb, int P, long long pixel_offset, 
       store_pe(PEb, wi, lane);
       __syncwarp();
       zero(acc);
-      warp_gemm<kPEPad>(PEb, sw + OFF_IW1P, acc, rg, cg);
+      warp_gemm<kPEPad - 4>(PEb, sw + OFF_IW1P, acc, rg, cg);
       store_relu_colbias(H1, acc, aP, rg, cg);
       __syncwarp();
       zero(acc);
       warp_gemm<kHidden>(H1, sw + OFF_IW2, acc, rg, cg);
       store_relu_colbias(H2, acc, sw + OFF_IB2, rg, cg);
+      const float dz1p = valid ? dz1 : 0.0f;
       DZ[lane] = dz0p;
-      DZ[32 + lane] = valid ? dz1 : 0.0f;
+      DZ[32 + lane] = dz1p;
+      gI.b3[0] += dz0p;
+      gI.b3[1] += dz1p;
       __syncwarp();
-      bwd_w3<2>(H2, DZ, sg + GI_W3, sg + GI_B3, lane);
+      bwd_out<2>(H2, DZ, sw + OFF_IW3, gI.w3, gI.b2, lane);
       __syncwarp();
-      bwd_head<2, 2>(H2, DZ, sw + OFF_IW3, H2, lane);   // dZ2 over H2, in place
-      __syncwarp();
-      bwd_weights(H1, 64, H2, sg + GI_W2, LD_2, 0, sg + GI_B2, lane);
-      __syncwarp();
-      bwd_hidden(H2, sw + OFF_IW2, H1, H1, lane);   // dZ1 over H1, in place
-      __syncwarp();
+      acc_w2(H1, H2, tacc, rg, cg);
+      bwd_hidden_tile(H2, sw + OFF_IW2T, H1, acc, rg, cg);
       store_pe(PEb, wi, lane);   // again, over the consumed dZ2
       __syncwarp();
-      bwd_weights(PEb, kPE, H1, sg + GI_W1, LD_I1, lf, sg + GI_B1, lane);
-      // the f part of layer 1 is shared by the chunk's rows: dW1f[c][k] += f[k] colsum(dZ1)[c]
-      // and dLoss/df[k] += sum_c colsum(dZ1)[c] W1f[k][c]
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int c = lane + 32 * h;
-        float cs = 0.0f;
-        for (int r = 0; r < 32; ++r) cs += H1[aidx(c, r)];
-        DZ[c] = cs;   // scratch: column sums of dZ1 (the output gradients are consumed)
-      }
-      __syncwarp();
-      for (int k = 0; k < lf; ++k) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int c = lane + 32 * h;
-          atomicAdd(sg + GI_W1 + c * LD_I1 + k, fP[k] * DZ[c]);
-        }
-      }
-      if (lane < lf) {
-        float s = 0.0f;
-        for (int c = 0; c < 64; ++c) s = fmaf(DZ[c], sw[OFF_IW1F + lane * 64 + c], s);
-        dfP[lane] += s;
-      }
+      acc_w1p(PEb, H1, tacc, rg, cg);
+      col_sums(H1, cs, lane);   // the f part of layer 1 is shared by the pixel's rows: once per pixel, below
       __syncwarp();
     }
+
+    DZ[own_col(lane, 0)] = cs[0];
+    DZ[own_col(lane, 1)] = cs[1];
+    gI.b1[0] += cs[0];
+    gI.b1[1] += cs[1];
+    __syncwarp();
+    const float dfk = bwd_shared_feature(fP, DZ, sw + OFF_IW1F, lf, g_irt, lane);
 
     // ---- primary encode adjoint: table gradients at x
     {
       const int l = lane >> 1;
-      if ((lane & 1) == 0 && l < m.grid.levels) encode_level_bwd(m.grid, l, x, dfP[lane], dfP[lane + 1], g_table, nullptr);
+      const float df1 = __shfl_down_sync(0xffffffffu, dfk, 1);
+      if ((lane & 1) == 0 && l < m.grid.levels) encode_level_bwd(m.grid, l, x, dfk, df1, g_table, nullptr);
     }
     __syncwarp();
   }
 
-  // ---- flush the CTA's weight gradients into the caller's blobs (canonical layouts)
-  __syncthreads();
-  flush_irt_grads(sg, m.lf, g_irt, kBT);
+  // ---- the CTA's gradients of I into the caller's blob, then give the tensor memory back
+  flush_irt_grads(sw + WADJ_FLOATS + WB_H1, WB_FLOATS, tacc, gI, lf, g_irt);
+  adj_tmem_free(tslot, threadIdx.x);
 }
 
 }  // namespace
@@ -354,9 +359,9 @@ cudaError_t prepare_backward_fp32() {
 
 cudaError_t launch_backward_fp32(const ModelDesc& m, const rt_gbuffer& gb, int P, long long offset, const float4* dL,
                                  float* g_table, float* g_brdf, float* g_irt, int num_sms, cudaStream_t s) {
-  const int need = (P + kBW - 1) / kBW;
+  const int need = (P + kAdjWarps - 1) / kAdjWarps;
   const int grid = need < num_sms ? need : num_sms;
-  backward_fp32_kernel<<<grid, kBT, kBSmem, s>>>(m, gb, P, offset, dL, g_table, g_brdf, g_irt);
+  backward_fp32_kernel<<<grid, kAdjThreads, kBSmem, s>>>(m, gb, P, offset, dL, g_table, g_brdf, g_irt);
   return cudaGetLastError();
 }
 

@@ -11,40 +11,37 @@
 //   (w . n > 0) and then over points.
 //
 // Work, in two phases of one persistent launch.  I phase: a unit is one
-// point and up to 128 of its directions; the warp encodes f = H(x), counts
-// the point's front-facing directions and walks the unit's directions 32 at
-// a time (lane = direction): I forward, the head gradients, I's adjoint with
-// the layer-1 f part shared by the rows; then it scatters the unit's share of
-// dLoss/df into the table (the encode adjoint is linear in it).  Splitting a
-// point's directions over units spreads a small batch (2048 points) over
-// every SM.  B phase: a warp takes 32 points as one 32-row tile (lane =
-// point), runs B, back-propagates the L1 of the BRDF heads and scatters the
-// B part of dLoss/df.  I's weight gradients go to the CTA's shared
-// accumulator and then to the caller's blob, B's straight to the caller's
-// blob (adjoint.cuh).
+// point and up to 256 of its directions; the warp encodes f = H(x), counts
+// the point's front-facing directions, lists the unit's (the others carry no
+// loss) and walks the list 32 at a time (lane = direction): I forward, the
+// head gradients, I's adjoint with the layer-1 f part shared by the unit's
+// rows; then it scatters the unit's share of dLoss/df into the table (the
+// encode adjoint is linear in it).  Splitting a point's directions over units
+// spreads a small batch (2048 points) over every SM.  B phase: a warp takes 32
+// points as one 32-row tile (lane = point), runs B, back-propagates the L1 of
+// the BRDF heads and scatters the B part of dLoss/df.  Where weight gradients
+// are summed: adjoint.cuh.
 #include "adjoint.cuh"
 
 namespace rtk {
 
 namespace {
 
-constexpr int kDW = 6;                      // warps per CTA (shared memory holds one CTA of 6 warps)
-constexpr int kUnitDirs = 128;              // directions of one point per I-phase work unit
-constexpr int kDT = 32 * kDW;
+constexpr int kUnitDirs = 256;              // directions of one point per I-phase work unit
 // per-warp buffers (floats)
 constexpr int DB_F = 0;                                    // f of the warp's 32 points [32 cols]
 constexpr int DB_H1 = DB_F + kActStride32;                 // layer-1 activations, then dZ1 (in place) [64 cols]
 // PE of the current directions [32 cols] for layer 1, then layer-2 activations and dZ2 (in place)
 // [64 cols]; the PE is written again for the PE part of dW1 once dZ2 is consumed
 constexpr int DB_H2 = DB_H1 + kActStride;
-constexpr int DB_DZ = DB_H2 + kActStride;                 // output gradients [8][32]
-constexpr int DB_FP = DB_DZ + 8 * 32;                      // f of the current point [32]
+constexpr int DB_DZ = DB_H2 + kActStride;                 // output gradients [7][32]; column sums [64]
+constexpr int DB_FP = DB_DZ + 7 * 32;                      // f of the current point [32]
 constexpr int DB_AP = DB_FP + 32;                          // b1 + W1f f of the current point [64]
-constexpr int DB_DFP = DB_AP + 64;                         // dLoss/df of the current point, I part [32]
-constexpr int DB_FLOATS = DB_DFP + 32;
-constexpr size_t kDSmem = (size_t)(WPACK_FLOATS + G_FLOATS + kDW * DB_FLOATS) * sizeof(float);
+constexpr int DB_LIST = DB_AP + 64;                        // the unit's front-facing directions, uint16 [256]
+constexpr int DB_FLOATS = DB_LIST + kUnitDirs / 2;
+constexpr size_t kDSmem = (size_t)(WADJ_FLOATS + kAdjWarps * DB_FLOATS + 4) * sizeof(float);
 static_assert(kDSmem <= 232448, "one CTA per SM");
-static_assert(DB_H1 % 4 == 0 && DB_H2 % 4 == 0 && DB_DZ % 4 == 0 &&
+static_assert(DB_H1 % 4 == 0 && DB_H2 % 4 == 0 && DB_H2 == DB_H1 + kActStride && DB_DZ % 4 == 0 &&
                   DB_FLOATS % 4 == 0,
               "float4 alignment");
 
@@ -68,22 +65,24 @@ __global__ void distill_dirs_kernel(long long PK, int K, int S, long long ray_of
   dirs[e] = make_float4(rho * cp, rho * sp, z, 0.0f);
 }
 
-__global__ void __launch_bounds__(kDT, 1)
+__global__ void __launch_bounds__(kAdjThreads, 1)
 distill_fp32_kernel(ModelDesc m, const float4* __restrict__ pos4, const float4* __restrict__ nrm4, int P, int K,
                     const float4* __restrict__ dirs, const float* __restrict__ brdf_t, const float* __restrict__ vis_t,
                     const float* __restrict__ depth_t, float* __restrict__ loss, float* __restrict__ g_table,
                     float* __restrict__ g_brdf, float* __restrict__ g_irt) {
   extern __shared__ float4 smem4[];
   float* sw = reinterpret_cast<float*>(smem4);
-  float* sg = sw + WPACK_FLOATS;
-  for (int i = threadIdx.x; i < WPACK_FLOATS / 4; i += kDT)
-    smem4[i] = __ldg(reinterpret_cast<const float4*>(m.wpack) + i);
-  for (int i = threadIdx.x; i < G_FLOATS; i += kDT) sg[i] = 0.0f;
-  __syncthreads();
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(sw + WADJ_FLOATS + kAdjWarps * DB_FLOATS);
+  load_adjoint_weights(sw, m.wpack);
+  const uint32_t tacc = adj_tmem_alloc(tslot, threadIdx.x);   // (its barrier also publishes the weights)
+  tmem_zero(tacc, 12);
+  IrtGrads gI;
+  zero(gI);
+  const float* bw = m.wpack;   // B's weights stay in global memory (one evaluation per point)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rg = lane >> 3, cg = lane & 7;
-  float* wb = sg + G_FLOATS + warp * DB_FLOATS;
+  float* wb = sw + WADJ_FLOATS + warp * DB_FLOATS;
   float* F = wb + DB_F;
   float* PEb = wb + DB_H2;   // shares H2's buffer (see DB_H2)
   float* H1 = wb + DB_H1;
@@ -91,7 +90,7 @@ distill_fp32_kernel(ModelDesc m, const float4* __restrict__ pos4, const float4* 
   float* DZ = wb + DB_DZ;
   float* fP = wb + DB_FP;
   float* aP = wb + DB_AP;
-  float* dfP = wb + DB_DFP;
+  uint16_t* list = reinterpret_cast<uint16_t*>(wb + DB_LIST);
   const int lf = m.lf, lfp = m.lfp, levels = m.grid.levels;
   const BlobB gB{g_brdf, lf};
   const float invR = 1.0f / (float)P;
@@ -101,7 +100,7 @@ distill_fp32_kernel(ModelDesc m, const float4* __restrict__ pos4, const float4* 
   // ---- I phase: units of (point, up to kUnitDirs of its directions), lane = direction
   const int nch = (K + kUnitDirs - 1) / kUnitDirs;
   const long long units = (long long)P * nch;
-  for (long long u = (long long)blockIdx.x * kDW + warp; u < units; u += (long long)gridDim.x * kDW) {
+  for (long long u = (long long)blockIdx.x * kAdjWarps + warp; u < units; u += (long long)gridDim.x * kAdjWarps) {
     {
       const int p = (int)(u / nch);
       const int kb = (int)(u - (long long)p * nch) * kUnitDirs;
@@ -119,7 +118,6 @@ distill_fp32_kernel(ModelDesc m, const float4* __restrict__ pos4, const float4* 
           fP[lane] = part.x;
           fP[lane + 1] = part.y;
         }
-        dfP[lane] = 0.0f;
       }
       __syncwarp();
 #pragma unroll
@@ -129,24 +127,31 @@ distill_fp32_kernel(ModelDesc m, const float4* __restrict__ pos4, const float4* 
         for (int k = 0; k < lfp; ++k) acc = fmaf(fP[k], sw[OFF_IW1F + k * 64 + c], acc);
         aP[c] = acc;
       }
-      int cnt = 0;
+      // the point's front-facing count, and the unit's front-facing directions in order: the others have no
+      // part in the loss, so only these are evaluated
+      int cnt = 0, nlist = 0;
       for (int k0 = 0; k0 < K; k0 += 32) {
         const int k = k0 + lane;
         const bool ff = k < K && dot(xyz(dirs[(size_t)p * K + k]), n) > 0.0f;
-        cnt += __popc(__ballot_sync(0xffffffffu, ff));
+        const unsigned bal = __ballot_sync(0xffffffffu, ff);
+        cnt += __popc(bal);
+        if (k0 >= kb && k0 < ke) {
+          if (ff) list[nlist + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(k - kb);
+          nlist += __popc(bal);
+        }
       }
       const float wI = cnt > 0 ? invR / (float)cnt : 0.0f;
+      float cs[2] = {0.f, 0.f};   // the unit's sum of dZ1, the lane's two columns
       __syncwarp();
-      for (int k0 = kb; k0 < ke; k0 += 32) {
-        const int k = k0 + lane;
-        const bool valid = k < ke;
-        const f3 w = valid ? xyz(dirs[(size_t)p * K + k]) : n;
-        const bool ff = valid && dot(w, n) > 0.0f;
-        float acc[8][8];
+      for (int r0 = 0; r0 < nlist; r0 += 32) {
+        const bool ff = r0 + lane < nlist;
+        const int k = kb + (int)list[ff ? r0 + lane : r0];
+        const f3 w = xyz(dirs[(size_t)p * K + k]);
+        Tile acc;
         store_pe(PEb, w, lane);
         __syncwarp();
         zero(acc);
-        warp_gemm<kPEPad>(PEb, sw + OFF_IW1P, acc, rg, cg);
+        warp_gemm<kPEPad - 4>(PEb, sw + OFF_IW1P, acc, rg, cg);
         store_relu_colbias(H1, acc, aP, rg, cg);
         __syncwarp();
         zero(acc);
@@ -168,54 +173,37 @@ distill_fp32_kernel(ModelDesc m, const float4* __restrict__ pos4, const float4* 
         }
         DZ[lane] = dz0;
         DZ[32 + lane] = dz1;
+        gI.b3[0] += dz0;
+        gI.b3[1] += dz1;
         __syncwarp();
-        bwd_w3<2>(H2, DZ, sg + GI_W3, sg + GI_B3, lane);
+        bwd_out<2>(H2, DZ, sw + OFF_IW3, gI.w3, gI.b2, lane);
         __syncwarp();
-        bwd_head<2, 2>(H2, DZ, sw + OFF_IW3, H2, lane);   // dZ2 over H2, in place
-        __syncwarp();
-        bwd_weights(H1, 64, H2, sg + GI_W2, LD_2, 0, sg + GI_B2, lane);
-        __syncwarp();
-        bwd_hidden(H2, sw + OFF_IW2, H1, H1, lane);   // dZ1 over H1, in place
-        __syncwarp();
+        acc_w2(H1, H2, tacc, rg, cg);
+        bwd_hidden_tile(H2, sw + OFF_IW2T, H1, acc, rg, cg);
         store_pe(PEb, w, lane);   // again, over the consumed dZ2
         __syncwarp();
-        bwd_weights(PEb, kPE, H1, sg + GI_W1, LD_I1, lf, sg + GI_B1, lane);
-        // the f part of layer 1 is shared by the rows: dW1f[c][k] += f[k] colsum(dZ1)[c],
-        // dLoss/df[k] += sum_c colsum(dZ1)[c] W1f[k][c]
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int c = lane + 32 * h;
-          float cs = 0.0f;
-          for (int r = 0; r < 32; ++r) cs += H1[aidx(c, r)];
-          DZ[c] = cs;   // scratch: column sums of dZ1 (the output gradients are consumed)
-        }
-        __syncwarp();
-        for (int kk = 0; kk < lf; ++kk) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int c = lane + 32 * h;
-            atomicAdd(sg + GI_W1 + c * LD_I1 + kk, fP[kk] * DZ[c]);
-          }
-        }
-        if (lane < lf) {
-          float s = 0.0f;
-          for (int c = 0; c < 64; ++c) s = fmaf(DZ[c], sw[OFF_IW1F + lane * 64 + c], s);
-          dfP[lane] += s;
-        }
+        acc_w1p(PEb, H1, tacc, rg, cg);
+        col_sums(H1, cs, lane);   // the f part of layer 1 is shared by the unit's rows: once per unit, below
         __syncwarp();
       }
-      {
+      if (nlist > 0) {
+        DZ[own_col(lane, 0)] = cs[0];
+        DZ[own_col(lane, 1)] = cs[1];
+        gI.b1[0] += cs[0];
+        gI.b1[1] += cs[1];
+        __syncwarp();
+        const float dfk = bwd_shared_feature(fP, DZ, sw + OFF_IW1F, lf, g_irt, lane);
         // the unit's share of dLoss/df (the encode adjoint is linear in it)
         const int l = lane >> 1;
-        if ((lane & 1) == 0 && l < levels)
-          encode_level_bwd(m.grid, l, x, dfP[lane], dfP[lane + 1], g_table, nullptr);
+        const float df1 = __shfl_down_sync(0xffffffffu, dfk, 1);
+        if ((lane & 1) == 0 && l < levels) encode_level_bwd(m.grid, l, x, dfk, df1, g_table, nullptr);
       }
       __syncwarp();
     }
   }
 
   // ---- B phase: groups of 32 points as one 32-row tile (lane = point)
-  for (int g0 = (blockIdx.x * kDW + warp) * 32; g0 < P; g0 += gridDim.x * kDW * 32) {
+  for (int g0 = (blockIdx.x * kAdjWarps + warp) * 32; g0 < P; g0 += gridDim.x * kAdjWarps * 32) {
     const int p = g0 + lane;
     const bool vp = p < P;
     {
@@ -228,22 +216,22 @@ distill_fp32_kernel(ModelDesc m, const float4* __restrict__ pos4, const float4* 
       }
     }
     __syncwarp();
-    float acc[8][8];
+    Tile acc;
     zero(acc);
-    warp_gemm_k(F, sw + OFF_BW1, acc, lfp, rg, cg);
-    store_relu_colbias(H1, acc, sw + OFF_BB1, rg, cg);
+    warp_gemm_k(F, bw + OFF_BW1, acc, lfp, rg, cg);
+    store_relu_colbias(H1, acc, bw + OFF_BB1, rg, cg);
     __syncwarp();
     zero(acc);
-    warp_gemm<kHidden>(H1, sw + OFF_BW2, acc, rg, cg);
-    store_relu_colbias(H2, acc, sw + OFF_BB2, rg, cg);
+    warp_gemm<kHidden>(H1, bw + OFF_BW2, acc, rg, cg);
+    store_relu_colbias(H2, acc, bw + OFF_BB2, rg, cg);
     __syncwarp();
     float y[7];
 #pragma unroll
-    for (int o = 0; o < 7; ++o) y[o] = sw[OFF_BB3 + o];
+    for (int o = 0; o < 7; ++o) y[o] = __ldg(bw + OFF_BB3 + o);
     for (int k = 0; k < kHidden; ++k) {
       const float hk = H2[aidx(k, lane)];
 #pragma unroll
-      for (int o = 0; o < 7; ++o) y[o] = fmaf(hk, sw[OFF_BW3 + 8 * k + o], y[o]);
+      for (int o = 0; o < 7; ++o) y[o] = fmaf(hk, __ldg(bw + OFF_BW3 + 8 * k + o), y[o]);
     }
     const float nlen = sqrtf(fmaxf(y[0] * y[0] + y[1] * y[1] + y[2] * y[2], 1e-24f));
     const f3 n2 = mk(y[0] / nlen, y[1] / nlen, y[2] / nlen);
@@ -278,17 +266,17 @@ distill_fp32_kernel(ModelDesc m, const float4* __restrict__ pos4, const float4* 
     __syncwarp();
     bwd_w3<7>(H2, DZ, gB.w3(), gB.b3(), lane, 64);
     __syncwarp();
-    bwd_head<7, 8>(H2, DZ, sw + OFF_BW3, H2, lane);   // dZ2 over H2, in place
+    bwd_head<7, 8>(H2, DZ, bw + OFF_BW3, H2, lane);   // dZ2 over H2, in place
     __syncwarp();
-    bwd_weights(H1, 64, H2, gB.w2(), 64, 0, gB.b2(), lane);
+    bwd_weights_global(H1, 64, H2, gB.w2(), 64, gB.b2(), lane);
     __syncwarp();
-    bwd_hidden(H2, sw + OFF_BW2, H1, H1, lane);   // dZ1 over H1, in place
+    bwd_hidden(H2, bw + OFF_BW2, H1, H1, lane);   // dZ1 over H1, in place
     __syncwarp();
-    bwd_weights(F, lf, H1, gB.w1(), lf, 0, gB.b1(), lane);
+    bwd_weights_global(F, lf, H1, gB.w1(), lf, gB.b1(), lane);
     float dF[32];
 #pragma unroll
     for (int k = 0; k < 32; ++k) dF[k] = 0.0f;
-    bwd_input(H1, sw + OFF_BW1, lf, dF, lane);
+    bwd_input(H1, bw + OFF_BW1, lf, dF, lane);
     {
       // segmented scatter over the warp's points (Morton order, runs of equal rows summed first)
       uint32_t dbits[32];
@@ -312,8 +300,8 @@ distill_fp32_kernel(ModelDesc m, const float4* __restrict__ pos4, const float4* 
     atomicAdd(loss + 1, l_bce);
     atomicAdd(loss + 2, l_depth);
   }
-  __syncthreads();
-  flush_irt_grads(sg, m.lf, g_irt, kDT);
+  flush_irt_grads(sw + WADJ_FLOATS + DB_H1, DB_FLOATS, tacc, gI, lf, g_irt);
+  adj_tmem_free(tslot, threadIdx.x);
 }
 
 __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m1,
@@ -348,9 +336,9 @@ cudaError_t launch_distill_fp32(const ModelDesc& m, const float4* pos, const flo
                                 float* loss, float* g_table, float* g_brdf, float* g_irt, int num_sms, cudaStream_t s) {
   const long long units = (long long)P * ((K + kUnitDirs - 1) / kUnitDirs);
   const long long groups = (P + 31) / 32;
-  const long long need = ((units > groups ? units : groups) + kDW - 1) / kDW;
+  const long long need = ((units > groups ? units : groups) + kAdjWarps - 1) / kAdjWarps;
   const int grid = (int)(need < num_sms ? need : num_sms);
-  distill_fp32_kernel<<<grid, kDT, kDSmem, s>>>(m, pos, nrm, P, K, dirs, brdf_t, vis_t, depth_t, loss, g_table,
+  distill_fp32_kernel<<<grid, kAdjThreads, kDSmem, s>>>(m, pos, nrm, P, K, dirs, brdf_t, vis_t, depth_t, loss, g_table,
                                                 g_brdf, g_irt);
   return cudaGetLastError();
 }

@@ -99,7 +99,7 @@ render_fp32_kernel(ModelDesc m, rt_gbuffer gb, int P, long long pixel_offset, fl
                           : cosine_direction(n, m.seed, dir_counter(q, M, 0));
 
       // (c) I(f, w_i)
-      float acc[8][8];
+      Tile acc;
       store_pe(actA, wi, lane);
       __syncwarp();
       zero(acc);
@@ -129,13 +129,15 @@ render_fp32_kernel(ModelDesc m, rt_gbuffer gb, int P, long long pixel_offset, fl
       zero(acc);
       warp_gemm_k(actA, sw + OFF_BW1, acc, lfp, rg, cg);
       store_relu_colbias(actB, acc, sw + OFF_BB1, rg, cg);
-      float a2b[8][8];
+      Tile a2b;
       zero(a2b);
       warp_gemm_k(actA, sw + OFF_IW1F, a2b, lfp, rg, cg);
 #pragma unroll
-      for (int r = 0; r < 8; ++r)
+      for (int c = 0; c < 8; ++c) {
+        const float b = sw[OFF_IB1 + ocol(cg, c)];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) a2b[r][c] += sw[OFF_IB1 + ocol(cg, c)];
+        for (int h = 0; h < 4; ++h) a2b.v[h][c] = make_float2(a2b.v[h][c].x + b, a2b.v[h][c].y + b);
+      }
       __syncwarp();
       zero(acc);
       warp_gemm<kHidden>(actB, sw + OFF_BW2, acc, rg, cg);

@@ -1,7 +1,7 @@
-"""The FP32 kernels where their tiles can go wrong: rows that fill no tile, tiles of many points.
+"""The FP32 kernels where their tiles can go wrong: rows that fill no tile, tiles of many points, several work units.
 
-Tolerances are those the same quantities have elsewhere (test_gpu_stages); the sizes put the edges of the 128-row tiles
-and of the per-point slots inside the data.
+Tolerances are those the same quantities have elsewhere (test_gpu_stages, test_gpu_distill); the sizes put the edges of
+the 128-row tiles, of the per-point slots and of the direction units inside the data.
 """
 import numpy as np
 import pytest
@@ -9,7 +9,7 @@ import torch
 
 import scenegen
 from oracle import mlp
-from tests import helpers
+from tests import helpers, test_gpu_distill
 
 pytestmark = pytest.mark.gpu
 
@@ -47,3 +47,9 @@ def test_mlp_rows(lib, P, K):
     np.testing.assert_allclose(out[:, 3:6], a.numpy(), atol=2e-6)
     np.testing.assert_allclose(out[:, 6], rr.numpy(), atol=2e-6)
     assert np.all(out[:, 7] == 0) and r.check() == 0
+
+
+# K = 1: points without a front-facing direction; K = 289, 576: two and three direction units, ragged
+@pytest.mark.parametrize("P, K", [(50, 1), (5, 289), (2, 576)])
+def test_distill_units(lib, P, K):
+    test_gpu_distill.test_distill_gradient_matches_oracle(lib, P, K)
