@@ -1,7 +1,7 @@
 """The FP32 kernels where their tiles can go wrong: rows that fill no tile, tiles of many points, several work units.
 
-Tolerances are those the same quantities have elsewhere (test_gpu_stages, test_gpu_distill); the sizes put the edges of
-the 128-row tiles, of the per-point slots and of the direction units inside the data.
+Tolerances are those the same quantities have elsewhere (test_gpu_render, test_gpu_stages, test_gpu_distill); the sizes put the edges of the 128-row tiles, of the per-pixel slots and of the direction units
+inside the data.
 """
 import numpy as np
 import pytest
@@ -9,6 +9,7 @@ import torch
 
 import scenegen
 from oracle import mlp
+from oracle import render as orender
 from tests import helpers, test_gpu_distill
 
 pytestmark = pytest.mark.gpu
@@ -20,6 +21,22 @@ def lib():
     build.build()
     from paper_2409_10327_gb300 import binding
     return binding
+
+
+# N < 4: more pixels in a tile than feature slots; 4: as many as there can be; 33, 130: pixels that start and end
+# anywhere in a tile and span several
+@pytest.mark.parametrize("n_dirs, P", [(1, 300), (2, 131), (3, 700), (4, 129), (33, 11), (130, 5)])
+def test_frame_tiles(lib, n_dirs, P):
+    cfg = helpers.small_cfg(n_dirs=n_dirs, m_dirs=3)
+    sc, gb = helpers.scene_arrays(cfg, 4, bias=0.2, n_pixels=P)
+    r = helpers.renderer_for(cfg, sc)
+    out = r.render_frame(helpers.to_cuda(gb), pixel_offset=17).cpu().numpy()
+    assert r.check() == 0
+    prm, opt = helpers.oracle_params(sc), helpers.oracle_options(cfg)
+    ref = orender.render(gb, prm, opt, pixel_offset=17)
+    sens = orender.float32_sensitivity(gb, prm, opt, pixel_offset=17, draws=4)
+    ok, stats = helpers.fp32_parity(out[:, :3], ref, sens)
+    assert ok, stats
 
 
 # rows = 1, 127, 128, 129 and one tile over the number of warpgroups; K = 1 and 3: more points in a tile than slots
