@@ -1,6 +1,7 @@
 """The FP32 kernels where their tiles can go wrong: rows that fill no tile, tiles of many points, several work units.
 
-Tolerances are those the same quantities have elsewhere (test_gpu_render, test_gpu_stages, test_gpu_distill); the sizes put the edges of the 128-row tiles, of the per-pixel slots and of the direction units
+Tolerances are those the same quantities have elsewhere (test_gpu_render, test_gpu_stages, test_gpu_distill,
+test_gpu_denoise); the sizes put the edges of the 128-row tiles, of the per-pixel slots and of the direction units
 inside the data.
 """
 import numpy as np
@@ -8,9 +9,10 @@ import pytest
 import torch
 
 import scenegen
+from oracle import denoise as oden
 from oracle import mlp
 from oracle import render as orender
-from tests import helpers, test_gpu_distill
+from tests import helpers, test_gpu_denoise, test_gpu_distill
 
 pytestmark = pytest.mark.gpu
 
@@ -70,3 +72,12 @@ def test_mlp_rows(lib, P, K):
 @pytest.mark.parametrize("P, K", [(50, 1), (5, 289), (2, 576)])
 def test_distill_units(lib, P, K):
     test_gpu_distill.test_distill_gradient_matches_oracle(lib, P, K)
+
+
+# images with and without blocks whose window lies inside, and every exponent's route
+@pytest.mark.parametrize("h, w, iters, sigma_n", [(26, 70, 2, 128.0), (17, 130, 1, 0.0), (40, 66, 1, 1.0), (33, 97, 2, 300.0)])
+def test_denoise_blocks(lib, h, w, iters, sigma_n):
+    c, z, n = test_gpu_denoise._image(h, w, h + w)
+    got = test_gpu_denoise._run(lib, c, z, n, iterations=iters, sigma_n=sigma_n)
+    ref_c, ref_v = oden.svgf(c, z, n, iterations=iters, sigma_n=sigma_n)
+    test_gpu_denoise._check(got, ref_c, ref_v)
