@@ -83,6 +83,7 @@ cudaError_t prepare_render_bf16() {
   e = e != cudaSuccess ? e : prepare_wg<4, false, false>();
   e = e != cudaSuccess ? e : prepare_wg<4, true, false>();
   e = e != cudaSuccess ? e : prepare_render_bf16_chunked();
+  e = e != cudaSuccess ? e : prepare_render_bf16_small();
   return e;
 }
 
@@ -102,8 +103,10 @@ cudaError_t launch_render_bf16_lights(const ModelDesc& m, const HeadParams& hp, 
     const float4* ee = envs + e0 * hw;
     float4* oo = out + (long long)e0 * P;
     const bool chunk = !m.hard && (m.dpt == 32 || m.dpt == 64) && m.N % m.dpt == 0 && m.N > m.dpt;
+    const int rep = m.hard ? 1 : small_replicas(P, m.N, num_sms);
     const cudaError_t err =
-        chunk       ? launch_render_bf16_chunked(nl, wg, mm, hp, gb, P, offset, ee, oo, num_sms, s)
+        rep > 1     ? launch_render_bf16_small(rep, nl, mm, hp, gb, P, offset, ee, oo, num_sms, s)
+        : chunk       ? launch_render_bf16_chunked(nl, wg, mm, hp, gb, P, offset, ee, oo, num_sms, s)
         : m.hard    ? launch_lights<4, true, false>(nl, mm, hp, gb, P, offset, ee, oo, num_sms, s)
         : wg == 2   ? launch_lights<2, false, false>(nl, mm, hp, gb, P, offset, ee, oo, num_sms, s)
         : wg == 3   ? launch_lights<3, false, false>(nl, mm, hp, gb, P, offset, ee, oo, num_sms, s)

@@ -72,6 +72,7 @@ constexpr int WG_BYTES_HARD = WG_CNT + 128;
 constexpr int SM_WG = WBF16_BYTES;
 static_assert(WG_MISC + 16 + kCarrySlots * 8 * 16 <= WG_BYTES, "warpgroup block overflow");
 static_assert(WG_CNT + 16 <= WG_BYTES_HARD, "warpgroup block overflow (hard visibility)");
+static_assert(64 * 64 <= 2 * kPixSlots * 64, "the replicas' exchanged features fit the slots");
 static_assert(128 * 16 <= 2 * kPixSlots * 64 && WG_MISC % 16 == 0 && WG_BYTES_HARD % 16 == 0, "pixel slots");
 
 template <int WG, bool HARD = false>
@@ -86,7 +87,7 @@ struct Layout {
   static constexpr int kCarveout = (int)((kMinBlocks * (kSmem + 1024) * 100 + 233471) / 233472);
 };
 
-template <int NL, int WG, bool HARD, bool CHUNK>
+template <int NL, int WG, bool HARD, bool CHUNK, int REP>
 __global__ void __launch_bounds__(Layout<WG, HARD>::kThreads, Layout<WG, HARD>::kMinBlocks)
 render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ HeadParams hp, rt_gbuffer gb, int P,
                    long long pixel_offset, const float4* __restrict__ envs, float4* __restrict__ out) {
@@ -383,10 +384,17 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
     // added in the same order, so the two orders give the same bits.
     // (the chunked order is compiled only into the CHUNK instantiations: in the others dpt is the
     // constant 0, which keeps the consecutive order's code as tight as without the option)
+    // REP > 1 (a launch whose warpgroups have no more than R = 128 / REP samples each): a tile holds R
+    // samples, each by REP rows, its replicas.  They share the sample's serial chain: each encodes
+    // 16 / REP levels of x' and takes every REP-th secondary direction, and the partial sums meet at
+    // the end, so the chain is 1 + 1 + M / REP evaluations long instead of 2 + M.
+    constexpr int R = 128 / REP;
+    static_assert(REP == 1 || (!HARD && !CHUNK), "replicas: the consecutive soft order only");
+    const int rep = REP > 1 ? t / R : 0, tr = REP > 1 ? t % R : t;
     const int dpt = CHUNK && (m.dpt == 32 || m.dpt == 64) && N % m.dpt == 0 && N > m.dpt ? m.dpt : 0;
     const int gpix = dpt ? 128 / dpt : 0;
     const int nchunk = dpt ? N / dpt : 1;
-    const long long ntiles = dpt ? (p1 - p0 + gpix - 1) / gpix * nchunk : (s_end - p0 * N + 127) / 128;
+    const long long ntiles = dpt ? (p1 - p0 + gpix - 1) / gpix * nchunk : (s_end - p0 * N + R - 1) / R;
     for (long long tile = 0; tile < ntiles; ++tile) {
       long long p_first, sbase = 0;
       int off0 = 0, nvalid, npix, chunk = 0;
@@ -396,14 +404,14 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
         npix = (int)min((long long)gpix, p1 - p_first);
         nvalid = npix * dpt;
       } else {
-        sbase = p0 * N + 128 * tile;
+        sbase = p0 * N + R * tile;
         p_first = sbase / N;
         off0 = (int)(sbase - p_first * N);
-        nvalid = (int)min(128LL, s_end - sbase);
+        nvalid = (int)min((long long)R, s_end - sbase);
         npix = (int)((sbase + nvalid - 1) / N - p_first) + 1;
       }
-      const bool valid = t < nvalid;
-      const int row = valid ? t : nvalid - 1;
+      const bool valid = tr < nvalid;
+      const int row = valid ? tr : nvalid - 1;
       int ps, i;
       if (dpt) {
         ps = row / dpt;
@@ -454,7 +462,7 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
       // this row is fr1 (v Lenv(w_i) + (1 - v) (pi/M) sum_j v'_j fr2_j Lenv(w'_j)).
       f3 c[NL];
       {
-        const f3 w0 = fr1 * v;
+        const f3 w0 = fr1 * (rep == 0 ? v : 0.0f);
         if (NL == 1) {
           c[0] = w0 * le1;
         } else {
@@ -464,7 +472,25 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
       }
 
       // (d) bounce: x' = x + t w_i; f' = H(x') into X columns 0..15
-      encode_point_tmem(m.grid, x + wi * tdep, X_w);
+      if constexpr (REP == 1) {
+        encode_point_tmem(m.grid, x + wi * tdep, X_w);
+      } else {
+        // the replicas' level groups meet in the feature slots, which the primary evaluation has consumed
+        uint32_t* fx = reinterpret_cast<uint32_t*>(fpix) + tr * 16;
+#pragma unroll
+        for (int k = 0; k < 4 / REP; ++k) {
+          const int it = rep * (4 / REP) + k;
+          uint32_t fq[4];
+          encode_group4(m.grid, x + wi * tdep, it, fq);
+          *reinterpret_cast<uint4*>(fx + 4 * it) = make_uint4(fq[0], fq[1], fq[2], fq[3]);
+        }
+        wg_sync(wg);
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+          const uint4 f = *reinterpret_cast<const uint4*>(fx + 4 * it);
+          tmem_st4(X_w + 4 * it, f.x, f.y, f.z, f.w);
+        }
+      }
       store_bias_cols_tmem(X_w);
 
       // (b) B(f')
@@ -486,7 +512,9 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
 
       // (c) + (e) at x': M directions about n'
       bool ok = true;
-      for (int j = 0; j < M && ok; ++j) {
+      for (int j0 = 0; j0 < M && ok; j0 += REP) {
+        const int j = REP > 1 ? min(j0 + rep, M - 1) : j0;
+        const bool own = REP == 1 || j0 + rep < M;   // a replica beyond the last direction repeats it with weight 0
         const f3 wj = cosine_direction_fast(n2, m.seed, dir_counter(q, M, 1 + j));
         const EnvTap tapj = env_tap_fast(m.env_h, m.env_w, wj);
         const f3 frw = fr1 * brdf_eval_fast(a2, r2, n2, wj, wo2, m.f0, m.lambert);
@@ -499,7 +527,7 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
         ok = run_mma([&] { mma_layer2(D_t, H_t, W_s + OFFB_IW2, W_s + OFFB_ONES, W_s + OFFB_IB2); });
         if (!ok) break;
         const float v2 = m.force_vis2 >= 0.f ? m.force_vis2 : sigmoid_fast(head_vis(D_w, hp.iw3v, hp.ib3[0]));
-        const f3 wj3 = frw * (wsec * v2);
+        const f3 wj3 = frw * (own ? wsec * v2 : 0.0f);
         if (NL == 1) {
           c[0] = c[0] + wj3 * lej;
         } else {
@@ -509,14 +537,30 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
       }
       if (!ok) break;
 
+      if constexpr (REP > 1) {   // the replicas' partial sums into replica 0's rows
+#pragma unroll
+        for (int e = 0; e < NL; ++e) {
+          wg_sync(wg);   // the exchanged features (first light) or the previous light's sums are read
+          red[t] = make_float4(c[e].x, c[e].y, c[e].z, 0.f);
+          wg_sync(wg);
+          if (rep == 0) {
+#pragma unroll
+            for (int k = 1; k < REP; ++k) {
+              const float4 h = red[t + R * k];
+              c[e] = mk(c[e].x + h.x, c[e].y + h.y, c[e].z + h.z);
+            }
+          }
+        }
+      }
+
       // deterministic segmented reduction of the tile's rows into their pixels,
       // one light at a time
-      const int key = valid ? ps : -1;
+      const int key = valid && rep == 0 ? ps : -1;
       const int prev = __shfl_up_sync(0xffffffffu, key, 1);
       const bool head = lane == 0 || prev != key;
   #pragma unroll
       for (int e = 0; e < NL; ++e) {
-        f3 ce = valid ? c[e] : mk(0.f, 0.f, 0.f);
+        f3 ce = key >= 0 ? c[e] : mk(0.f, 0.f, 0.f);
   #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
           const float ox = __shfl_down_sync(0xffffffffu, ce.x, off);
@@ -570,44 +614,44 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
                  : "memory");
 }
 
-template <int NL, int WG, bool HARD, bool CHUNK>
+template <int NL, int WG, bool HARD, bool CHUNK, int REP>
 cudaError_t prepare_variant() {
   using L = Layout<WG, HARD>;
-  cudaError_t e = cudaFuncSetAttribute(render_bf16_kernel<NL, WG, HARD, CHUNK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(render_bf16_kernel<NL, WG, HARD, CHUNK, REP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)L::kSmem);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(render_bf16_kernel<NL, WG, HARD, CHUNK>, cudaFuncAttributePreferredSharedMemoryCarveout,
+  return cudaFuncSetAttribute(render_bf16_kernel<NL, WG, HARD, CHUNK, REP>, cudaFuncAttributePreferredSharedMemoryCarveout,
                               L::kCarveout);
 }
 
-template <int NL, int WG, bool HARD, bool CHUNK>
+template <int NL, int WG, bool HARD, bool CHUNK, int REP>
 cudaError_t launch_variant(const ModelDesc& m, const HeadParams& hp, const rt_gbuffer& gb, int P, long long offset,
                            const float4* envs, float4* out, int num_sms, cudaStream_t s) {
   using L = Layout<WG, HARD>;
   const long long per_sm = L::kMinBlocks;
   const long long want = ((long long)P + WG - 1) / WG;
   const int grid = (int)(want < per_sm * num_sms ? want : per_sm * num_sms);
-  render_bf16_kernel<NL, WG, HARD, CHUNK><<<grid, L::kThreads, L::kSmem, s>>>(m, hp, gb, P, offset, envs, out);
+  render_bf16_kernel<NL, WG, HARD, CHUNK, REP><<<grid, L::kThreads, L::kSmem, s>>>(m, hp, gb, P, offset, envs, out);
   return cudaGetLastError();
 }
 
-template <int WG, bool HARD, bool CHUNK>
+template <int WG, bool HARD, bool CHUNK, int REP = 1>
 cudaError_t launch_lights(int nl, const ModelDesc& m, const HeadParams& hp, const rt_gbuffer& gb, int P,
                           long long offset, const float4* envs, float4* out, int num_sms, cudaStream_t s) {
   switch (nl) {
-    case 8: return launch_variant<8, WG, HARD, CHUNK>(m, hp, gb, P, offset, envs, out, num_sms, s);
-    case 4: return launch_variant<4, WG, HARD, CHUNK>(m, hp, gb, P, offset, envs, out, num_sms, s);
-    case 2: return launch_variant<2, WG, HARD, CHUNK>(m, hp, gb, P, offset, envs, out, num_sms, s);
-    default: return launch_variant<1, WG, HARD, CHUNK>(m, hp, gb, P, offset, envs, out, num_sms, s);
+    case 8: return launch_variant<8, WG, HARD, CHUNK, REP>(m, hp, gb, P, offset, envs, out, num_sms, s);
+    case 4: return launch_variant<4, WG, HARD, CHUNK, REP>(m, hp, gb, P, offset, envs, out, num_sms, s);
+    case 2: return launch_variant<2, WG, HARD, CHUNK, REP>(m, hp, gb, P, offset, envs, out, num_sms, s);
+    default: return launch_variant<1, WG, HARD, CHUNK, REP>(m, hp, gb, P, offset, envs, out, num_sms, s);
   }
 }
 
-template <int WG, bool HARD, bool CHUNK>
+template <int WG, bool HARD, bool CHUNK, int REP = 1>
 cudaError_t prepare_wg() {
-  cudaError_t e = prepare_variant<1, WG, HARD, CHUNK>();
-  e = e != cudaSuccess ? e : prepare_variant<2, WG, HARD, CHUNK>();
-  e = e != cudaSuccess ? e : prepare_variant<4, WG, HARD, CHUNK>();
-  e = e != cudaSuccess ? e : prepare_variant<8, WG, HARD, CHUNK>();
+  cudaError_t e = prepare_variant<1, WG, HARD, CHUNK, REP>();
+  e = e != cudaSuccess ? e : prepare_variant<2, WG, HARD, CHUNK, REP>();
+  e = e != cudaSuccess ? e : prepare_variant<4, WG, HARD, CHUNK, REP>();
+  e = e != cudaSuccess ? e : prepare_variant<8, WG, HARD, CHUNK, REP>();
   return e;
 }
 

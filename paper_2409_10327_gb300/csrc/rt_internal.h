@@ -137,6 +137,12 @@ cudaError_t prepare_render_bf16_chunked();
 cudaError_t launch_render_bf16_chunked(int nl, int wg, const ModelDesc& m, const HeadParams& hp, const rt_gbuffer& gb,
                                        int P, long long offset, const float4* envs, float4* out, int num_sms,
                                        cudaStream_t s);
+// launches too small to fill 128-row tiles, soft visibility, one launch of nl lights: rep = small_replicas() > 1
+cudaError_t prepare_render_bf16_small();
+int small_replicas(int P, int N, int num_sms);
+cudaError_t launch_render_bf16_small(int rep, int nl, const ModelDesc& m, const HeadParams& hp, const rt_gbuffer& gb,
+                                     int P, long long offset, const float4* envs, float4* out, int num_sms,
+                                     cudaStream_t s);
 cudaError_t launch_render_bf16_lights(const ModelDesc& m, const HeadParams& hp, const rt_gbuffer& gb, int P,
                                       long long offset, const float4* envs, int E, float4* out, int num_sms,
                                       int max_nl, int wg, cudaStream_t s);

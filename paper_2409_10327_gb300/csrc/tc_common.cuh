@@ -275,66 +275,71 @@ __device__ __forceinline__ float head_vis(uint32_t taddr, const float* w, float 
 // the tile's 128 rows; halved so that it always fits half precision when the
 // table is FP16).  The adjoint's dLoss/dx' then needs no second gather.
 template <bool JAC = false>
+__device__ __forceinline__ void encode_group4(const GridDesc& g, f3 x, int it, uint32_t (&fq)[4], uint32_t* jac = nullptr,
+                                              int row = 0) {
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const int l = 4 * it + b;
+    float f0 = 0.f, f1 = 0.f;
+    if (l < g.levels) {
+      const int res = g.res[l];
+      uint32_t ix, iy, iz;
+      float w[3];
+      grid_cell(x.x, res, ix, w[0]);
+      grid_cell(x.y, res, iy, w[1]);
+      grid_cell(x.z, res, iz, w[2]);
+      const uint32_t* tab = reinterpret_cast<const uint32_t*>(g.table) + ((size_t)l << g.log2T);
+      const int dn = g.dense[l];
+      uint32_t v[8];
+#pragma unroll
+      for (int yz = 0; yz < 4; ++yz) {
+        const uint32_t r0 = corner_row(ix, iy + (yz & 1), iz + (yz >> 1), res, dn, g.mask);
+        const uint32_t r1 = corner_row(ix + 1, iy + (yz & 1), iz + (yz >> 1), res, dn, g.mask);
+        const uint2 pr = __ldg(reinterpret_cast<const uint2*>(tab + (r0 & ~1u)));
+        const bool odd = r0 & 1u;
+        v[2 * yz] = odd ? pr.y : pr.x;
+        v[2 * yz + 1] = ((r0 ^ r1) == 1u) ? (odd ? pr.x : pr.y) : __ldg(tab + r1);
+      }
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        // v[2*yz + dx] holds corner (dx, yz & 1, yz >> 1)
+        const int dx = c & 1, yz = c >> 1;
+        const float wt = (dx ? w[0] : 1.0f - w[0]) * ((yz & 1) ? w[1] : 1.0f - w[1]) *
+                         ((yz & 2) ? w[2] : 1.0f - w[2]);
+        const float2 e = __half22float2(*reinterpret_cast<const __half2*>(&v[c]));
+        f0 = fmaf(wt, e.x, f0);
+        f1 = fmaf(wt, e.y, f1);
+      }
+      if constexpr (JAC) {
+        float2 j[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const int cx = c & 1, cy = (c >> 1) & 1, cz = c >> 2;   // corner c = v[c] (x fastest)
+          const float2 e = __half22float2(*reinterpret_cast<const __half2*>(&v[c]));
+          const float ax = cx ? w[0] : 1.0f - w[0], ay = cy ? w[1] : 1.0f - w[1], az = cz ? w[2] : 1.0f - w[2];
+          const float gx = (cx ? 0.5f : -0.5f) * ay * az, gy = (cy ? 0.5f : -0.5f) * ax * az,
+                      gz = (cz ? 0.5f : -0.5f) * ax * ay;
+          j[0] = make_float2(fmaf(gx, e.x, j[0].x), fmaf(gx, e.y, j[0].y));
+          j[1] = make_float2(fmaf(gy, e.x, j[1].x), fmaf(gy, e.y, j[1].y));
+          j[2] = make_float2(fmaf(gz, e.x, j[2].x), fmaf(gz, e.y, j[2].y));
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const __half2 h = __floats2half2_rn(j[a].x, j[a].y);
+          jac[(3 * l + a) * 128 + row] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+      }
+    }
+    fq[b] = pack_bf16(f0, f1);
+  }
+}
+template <bool JAC = false>
 __device__ __forceinline__ void encode_point_tmem(const GridDesc& g, f3 x, uint32_t x_taddr, uint32_t* jac = nullptr,
                                                   int row = 0) {
 #pragma unroll 1
   for (int it = 0; it < kMaxLevels / 4; ++it) {
     uint32_t fq[4];
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int l = 4 * it + b;
-      float f0 = 0.f, f1 = 0.f;
-      if (l < g.levels) {
-        const int res = g.res[l];
-        uint32_t ix, iy, iz;
-        float w[3];
-        grid_cell(x.x, res, ix, w[0]);
-        grid_cell(x.y, res, iy, w[1]);
-        grid_cell(x.z, res, iz, w[2]);
-        const uint32_t* tab = reinterpret_cast<const uint32_t*>(g.table) + ((size_t)l << g.log2T);
-        const int dn = g.dense[l];
-        uint32_t v[8];
-#pragma unroll
-        for (int yz = 0; yz < 4; ++yz) {
-          const uint32_t r0 = corner_row(ix, iy + (yz & 1), iz + (yz >> 1), res, dn, g.mask);
-          const uint32_t r1 = corner_row(ix + 1, iy + (yz & 1), iz + (yz >> 1), res, dn, g.mask);
-          const uint2 pr = __ldg(reinterpret_cast<const uint2*>(tab + (r0 & ~1u)));
-          const bool odd = r0 & 1u;
-          v[2 * yz] = odd ? pr.y : pr.x;
-          v[2 * yz + 1] = ((r0 ^ r1) == 1u) ? (odd ? pr.x : pr.y) : __ldg(tab + r1);
-        }
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          // v[2*yz + dx] holds corner (dx, yz & 1, yz >> 1)
-          const int dx = c & 1, yz = c >> 1;
-          const float wt = (dx ? w[0] : 1.0f - w[0]) * ((yz & 1) ? w[1] : 1.0f - w[1]) *
-                           ((yz & 2) ? w[2] : 1.0f - w[2]);
-          const float2 e = __half22float2(*reinterpret_cast<const __half2*>(&v[c]));
-          f0 = fmaf(wt, e.x, f0);
-          f1 = fmaf(wt, e.y, f1);
-        }
-        if constexpr (JAC) {
-          float2 j[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            const int cx = c & 1, cy = (c >> 1) & 1, cz = c >> 2;   // corner c = v[c] (x fastest)
-            const float2 e = __half22float2(*reinterpret_cast<const __half2*>(&v[c]));
-            const float ax = cx ? w[0] : 1.0f - w[0], ay = cy ? w[1] : 1.0f - w[1], az = cz ? w[2] : 1.0f - w[2];
-            const float gx = (cx ? 0.5f : -0.5f) * ay * az, gy = (cy ? 0.5f : -0.5f) * ax * az,
-                        gz = (cz ? 0.5f : -0.5f) * ax * ay;
-            j[0] = make_float2(fmaf(gx, e.x, j[0].x), fmaf(gx, e.y, j[0].y));
-            j[1] = make_float2(fmaf(gy, e.x, j[1].x), fmaf(gy, e.y, j[1].y));
-            j[2] = make_float2(fmaf(gz, e.x, j[2].x), fmaf(gz, e.y, j[2].y));
-          }
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            const __half2 h = __floats2half2_rn(j[a].x, j[a].y);
-            jac[(3 * l + a) * 128 + row] = *reinterpret_cast<const uint32_t*>(&h);
-          }
-        }
-      }
-      fq[b] = pack_bf16(f0, f1);
-    }
+    encode_group4<JAC>(g, x, it, fq, jac, row);
     tmem_st4(x_taddr + 4 * it, fq[0], fq[1], fq[2], fq[3]);
   }
 }
