@@ -202,9 +202,11 @@ distill_fp32_kernel(ModelDesc m, const float4* __restrict__ pos4, const float4* 
     }
   }
 
-  // ---- B phase: groups of 32 points as one 32-row tile (lane = point)
-  for (int g0 = (blockIdx.x * kAdjWarps + warp) * 32; g0 < P; g0 += gridDim.x * kAdjWarps * 32) {
-    const int p = g0 + lane;
+  // ---- B phase: groups of 32 points as one 32-row tile (lane = point), from the last warp on: the first ones may
+  // have had one unit more
+  for (long long g0 = ((long long)(gridDim.x - blockIdx.x) * kAdjWarps - 1 - warp) * 32; g0 < P;
+       g0 += (long long)gridDim.x * kAdjWarps * 32) {
+    const int p = (int)min(g0 + lane, (long long)P);
     const bool vp = p < P;
     {
       const f3 x = vp ? xyz(pos4[p]) : mk(0.f, 0.f, 0.f);

@@ -141,7 +141,7 @@ render_fp32_kernel(const __grid_constant__ ModelDesc m, rt_gbuffer gb, int P, lo
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x;
-  const int wg = tid >> 7, t = tid & 127, warp = t >> 5, lane = t & 31;
+  const int wg = __shfl_sync(0xffffffffu, tid >> 7, 0), t = tid & 127, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane = t & 31;
   const int rg = lane >> 3, cg = lane & 7;
   uint8_t* wgb = sm + SM_WG + wg * WG_BYTES;
   float* aP = reinterpret_cast<float*>(wgb + WG_AP);
@@ -175,7 +175,7 @@ render_fp32_kernel(const __grid_constant__ ModelDesc m, rt_gbuffer gb, int P, lo
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot + (uint32_t)(256 * wg);
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0) + (uint32_t)(256 * wg);
   const uint32_t D_t = tmem + TM_D, X_t = tmem + TM_X, H_t = tmem + TM_H;   // MMA operands (lane 0)
   const uint32_t lane_off = (uint32_t)(32 * warp) << 16;                    // this warp's 32 lanes
   const uint32_t D_w = D_t + lane_off, X_w = X_t + lane_off, H_w = H_t + lane_off;
@@ -203,10 +203,12 @@ render_fp32_kernel(const __grid_constant__ ModelDesc m, rt_gbuffer gb, int P, lo
     tc_fence_before();
     abort = wg_sync_or(wg, abort);
     if (abort) return false;
-    if (t == 0) {
+    if (warp == 0) {
+      const uint32_t one = elect_one();
       tc_fence_after();
-      chain();
-      mma_commit(bar);
+      chain(one);
+      mma_commit_one(one, bar);
+      __syncwarp();
     }
     return true;
   };
@@ -219,8 +221,8 @@ render_fp32_kernel(const __grid_constant__ ModelDesc m, rt_gbuffer gb, int P, lo
     phase ^= 1u;
     tc_fence_after();
   };
-  auto irt_layer1 = [&] { return issue([&] { mma_split3<0, 4>(D_t, X_t, S + SM_W1); }); };
-  auto irt_layer2 = [&] { return issue([&] { mma_split3_layer2(D_t, H_t, S + SM_W2, S + SM_ONES, S + SM_B2); }); };
+  auto irt_layer1 = [&] { return issue([&](uint32_t one) { mma_split3<0, 4>(one, D_t, X_t, S + SM_W1); }); };
+  auto irt_layer2 = [&] { return issue([&](uint32_t one) { mma_split3_layer2(one, D_t, H_t, S + SM_W2, S + SM_ONES, S + SM_B2); }); };
 
   uint32_t parity = 0;
   for (long long sbase = p0 * N; sbase < s_end; sbase += 128, parity ^= 1u) {

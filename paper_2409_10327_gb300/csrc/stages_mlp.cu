@@ -44,7 +44,7 @@ mlp_rows_kernel(const __grid_constant__ ModelDesc m, const float* __restrict__ f
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x;
-  const int wg = tid >> 7, t = tid & 127, warp = t >> 5;
+  const int wg = __shfl_sync(0xffffffffu, tid >> 7, 0), t = tid & 127, warp = __shfl_sync(0xffffffffu, t >> 5, 0);
   uint8_t* slots = sm + SM_WG + wg * WG_BYTES;
   const float* hd = reinterpret_cast<const float*>(sm + SM_HEAD);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + kTmemSlot);
@@ -74,7 +74,7 @@ mlp_rows_kernel(const __grid_constant__ ModelDesc m, const float* __restrict__ f
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot + (uint32_t)(256 * wg);
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0) + (uint32_t)(256 * wg);
   const uint32_t D_t = tmem + TM_D, X_t = tmem + TM_X, H_t = tmem + TM_H;
   const uint32_t lane_off = (uint32_t)(32 * warp) << 16;
   const uint32_t D_w = D_t + lane_off, X_w = X_t + lane_off, H_w = H_t + lane_off;
@@ -89,10 +89,12 @@ mlp_rows_kernel(const __grid_constant__ ModelDesc m, const float* __restrict__ f
     tc_fence_before();
     abort = wg_sync_or(wg, abort);
     if (abort) return false;
-    if (t == 0) {
+    if (warp == 0) {
+      const uint32_t one = elect_one();
       tc_fence_after();
-      chain();
-      mma_commit(bar);
+      chain(one);
+      mma_commit_one(one, bar);
+      __syncwarp();
     }
     return true;
   };
@@ -159,14 +161,14 @@ mlp_rows_kernel(const __grid_constant__ ModelDesc m, const float* __restrict__ f
   long long tile = (long long)blockIdx.x * kWG + wg;
   if (tile < ntiles) load_tile(tile);
   for (; tile < ntiles; tile += stride) {
-    if (!issue([&] {
-          if (IRT) mma_split3<0, 4>(D_t, X_t, S + SM_W1);
-          else mma_split3_brdf1(D_t, X_t, S + SM_W1);
+    if (!issue([&](uint32_t one) {
+          if (IRT) mma_split3<0, 4>(one, D_t, X_t, S + SM_W1);
+          else mma_split3_brdf1(one, D_t, X_t, S + SM_W1);
         }))
       break;
     wait();
     epilogue_split3(D_w, H_w);
-    if (!issue([&] { mma_split3_layer2(D_t, H_t, S + SM_W2, S + SM_ONES, S + SM_B2); })) break;
+    if (!issue([&](uint32_t one) { mma_split3_layer2(one, D_t, H_t, S + SM_W2, S + SM_ONES, S + SM_B2); })) break;
     if (tile + stride < ntiles) load_tile(tile + stride);
     wait();
     const long long r = tile * 128 + t;
