@@ -161,22 +161,22 @@ __device__ __forceinline__ void slice_add_mapped(const uint8_t* slice, float* ds
 }
 
 // dW (+ db) of one layer over the tile: G[0:64) <- A^T B over the 128 rows, G[64:80) <- A^T ones.
-__device__ __forceinline__ void mma_weight_grad(uint32_t g, uint32_t sa, uint32_t sb, uint32_t ones) {
+__device__ __forceinline__ void mma_weight_grad(uint32_t one, uint32_t g, uint32_t sa, uint32_t sb, uint32_t ones) {
 #pragma unroll
-  for (int k = 0; k < 8; ++k) mma_bf16(g, sdesc_mn(sa + 2048 * k), sdesc_mn(sb + 2048 * k), kIdescDW, k > 0 ? 1u : 0u);
+  for (int k = 0; k < 8; ++k) mma_bf16(one, g, sdesc_mn(sa + 2048 * k), sdesc_mn(sb + 2048 * k), kIdescDW, k > 0 ? 1u : 0u);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) mma_bf16(g + 64, sdesc_mn(sa + 2048 * k), sdesc_mn32(ones + 512 * k), kIdescDB, k > 0 ? 1u : 0u);
+  for (int k = 0; k < 8; ++k) mma_bf16(one, g + 64, sdesc_mn(sa + 2048 * k), sdesc_mn32(ones + 512 * k), kIdescDB, k > 0 ? 1u : 0u);
 }
 // dW3^T over the tile: G[80:96) <- relu(pre2)^T dZ3 (rows = hidden units, columns = outputs)
-__device__ __forceinline__ void mma_w3_grad(uint32_t g, uint32_t sc, uint32_t sd) {
+__device__ __forceinline__ void mma_w3_grad(uint32_t one, uint32_t g, uint32_t sc, uint32_t sd) {
 #pragma unroll
-  for (int k = 0; k < 8; ++k) mma_bf16(g + 80, sdesc_mn(sc + 2048 * k), sdesc_mn32(sd + 512 * k), kIdescDB, k > 0 ? 1u : 0u);
+  for (int k = 0; k < 8; ++k) mma_bf16(one, g + 80, sdesc_mn(sc + 2048 * k), sdesc_mn32(sd + 512 * k), kIdescDB, k > 0 ? 1u : 0u);
 }
 // D <- Z . W^T: Z (the rows' dZ, bf16) in tensor memory, W the forward's weight tile [out][in]
 // (K-major for the forward) read MN-major, i.e. as W^T [in][out]; N = 64 (all inputs) or 32 (f)
-__device__ __forceinline__ void mma_input_grad(uint32_t d, uint32_t z_t, uint32_t w_s, uint32_t idesc, uint32_t acc0) {
+__device__ __forceinline__ void mma_input_grad(uint32_t one, uint32_t d, uint32_t z_t, uint32_t w_s, uint32_t idesc, uint32_t acc0) {
 #pragma unroll
-  for (int k = 0; k < 4; ++k) mma_bf16_ts(d, z_t + 8 * k, sdesc_mn(w_s + 2048 * k), idesc, (k > 0 || acc0) ? 1u : 0u);
+  for (int k = 0; k < 4; ++k) mma_bf16_ts(one, d, z_t + 8 * k, sdesc_mn(w_s + 2048 * k), idesc, (k > 0 || acc0) ? 1u : 0u);
 }
 
 // The primary evaluation's layer-1 input [f | PE(w) | 1 | 1 | 0] as bf16 hi parts into X (the
@@ -209,7 +209,8 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x;
-  const int wg = tid >> 7, t = tid & 127, warp = t >> 5, lane = t & 31;
+  const int wg = __shfl_sync(0xffffffffu, tid >> 7, 0), t = tid & 127, lane = t & 31;
+  const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);   // warp-uniform, as is what the MMA issue takes
   uint8_t* Wsm = sm + BS_W;
   uint8_t* wgb = sm + BS_WGB + wg * WB_BYTES;
   uint8_t* SA = wgb + WB_SA;
@@ -237,7 +238,7 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot + (uint32_t)(256 * wg);
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0) + (uint32_t)(256 * wg);
   const uint32_t D_t = tmem + BT_D, X_t = tmem + BT_X, H_t = tmem + BT_H, G_t = tmem + BT_G, F_t = tmem + BT_F;
   const uint32_t lane_off = (uint32_t)(32 * warp) << 16;
   const uint32_t D_w = D_t + lane_off, X_w = X_t + lane_off, H_w = H_t + lane_off, G_w = G_t + lane_off,
@@ -274,10 +275,12 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
     tc_fence_before();
     abort = wg_sync_or(wg, abort);
     if (abort) return false;
-    if (t == 0) {
+    if (warp == 0) {
+      const uint32_t one = elect_one();
       tc_fence_after();
-      issue();
-      mma_commit(bar_a);
+      issue(one);
+      mma_commit(one, bar_a);
+      __syncwarp();
     }
     if (!mbar_wait(bar_a, phase)) {
       if (!abort && t == 0) atomicOr(m.status, kStatusTimeout | 2u);
@@ -378,10 +381,10 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
       for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
       if (lane == 0) atomicAdd(gb3 + o, v);
     }
-    if (!run_mma([&] {
-          mma_input_grad(D_t, H_t, w2s, kIdescT64, 0u);
-          mma_weight_grad(G_t, SA_s, SB_s, ONES_s);
-          mma_w3_grad(G_t, SC_s, SD_s);
+    if (!run_mma([&](uint32_t one) {
+          mma_input_grad(one, D_t, H_t, w2s, kIdescT64, 0u);
+          mma_weight_grad(one, G_t, SA_s, SB_s, ONES_s);
+          mma_w3_grad(one, G_t, SC_s, SD_s);
         }))
       return false;
     const int grow = 16 * warp + lane;   // the G row of lanes 0..15
@@ -423,9 +426,9 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
 #pragma unroll
       for (int k = 0; k < 4; ++k) stage_chunk(SB, t, 4 * h + k, r[4 * k], r[4 * k + 1], r[4 * k + 2], r[4 * k + 3]);
     }
-    if (!run_mma([&] {
-          mma_input_grad(F_t, H_t, w1s, kIdescT32, acc_f ? 1u : 0u);
-          mma_weight_grad(G_t, SA_s, SB_s, ONES_s);
+    if (!run_mma([&](uint32_t one) {
+          mma_input_grad(one, F_t, H_t, w1s, kIdescT32, acc_f ? 1u : 0u);
+          mma_weight_grad(one, G_t, SA_s, SB_s, ONES_s);
         }))
       return false;
     // dW1 (the ones columns of the input are not mapped; db1 is column 64)
@@ -471,10 +474,10 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
 
     // (c) I(f, w_i) in split precision, as the forward: v and t
     store_primary_split(fpix, ps, X_w, H_w, wi);
-    if (!run_mma([&] { mma_layer1_split(D_t, X_t, H_t, W_s + OFFB_IW1, W_s + OFFB_IW1L); })) break;
+    if (!run_mma([&](uint32_t one) { mma_layer1_split(one, D_t, X_t, H_t, W_s + OFFB_IW1, W_s + OFFB_IW1L); })) break;
     epilogue_hidden_split(D_w, X_w, H_w);
-    if (!run_mma([&] {
-          mma_layer2_split(D_t, X_t, H_t, W_s + OFFB_IW2, W_s + OFFB_IW2L, W_s + OFFB_ONES, W_s + OFFB_IB2);
+    if (!run_mma([&](uint32_t one) {
+          mma_layer2_split(one, D_t, X_t, H_t, W_s + OFFB_IW2, W_s + OFFB_IW2L, W_s + OFFB_ONES, W_s + OFFB_IB2);
         }))
       break;
     float z0p, z1p;
@@ -492,9 +495,9 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
     // (d) f' = H(x') into X, with its derivative along the cell fractions for dLoss/dx'; (b) B(f')
     encode_point_tmem<true>(m.grid, x2, X_w, jac, t);
     store_bias_cols_tmem(X_w);
-    if (!run_mma([&] { mma_brdf_layer1(D_t, X_t, W_s + OFFB_BW1); })) break;
+    if (!run_mma([&](uint32_t one) { mma_brdf_layer1(one, D_t, X_t, W_s + OFFB_BW1); })) break;
     epilogue_hidden(D_w, H_w);
-    if (!run_mma([&] { mma_layer2(D_t, H_t, W_s + OFFB_BW2, W_s + OFFB_ONES, W_s + OFFB_BB2); })) break;
+    if (!run_mma([&](uint32_t one) { mma_layer2(one, D_t, H_t, W_s + OFFB_BW2, W_s + OFFB_ONES, W_s + OFFB_BB2); })) break;
     float yB[7];
     head_fp32<7, 8>(D_w, &hp.bw3[0][0], hp.bb3, yB);
     const float nlen = sqrtf(fmaxf(yB[0] * yB[0] + yB[1] * yB[1] + yB[2] * yB[2], 1e-24f));
@@ -523,10 +526,10 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
       const f3 fr2 = mk(a2.x * kInvPi + s, a2.y * kInvPi + s, a2.z * kInvPi + s);
       const f3 ef = le * fr2;
       store_pe_tmem(X_w, wj);
-      ok = run_mma([&] { mma_layer1(D_t, X_t, W_s + OFFB_IW1); });
+      ok = run_mma([&](uint32_t one) { mma_layer1(one, D_t, X_t, W_s + OFFB_IW1); });
       if (!ok) break;
       epilogue_hidden(D_w, H_w);
-      ok = run_mma([&] { mma_layer2(D_t, H_t, W_s + OFFB_IW2, W_s + OFFB_ONES, W_s + OFFB_IB2); });
+      ok = run_mma([&](uint32_t one) { mma_layer2(one, D_t, H_t, W_s + OFFB_IW2, W_s + OFFB_ONES, W_s + OFFB_IB2); });
       if (!ok) break;
       const float z0 = head_vis(D_w, hp.iw3v, hp.ib3[0]);
       const float v2 = m.force_vis2 >= 0.f ? m.force_vis2 : sigmoid_fast(z0);
@@ -548,9 +551,9 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
 
     // B backward (forward recomputed: the secondary loop overwrote D and H)
     store_bias_cols_tmem(X_w);
-    if (!run_mma([&] { mma_brdf_layer1(D_t, X_t, W_s + OFFB_BW1); })) break;
+    if (!run_mma([&](uint32_t one) { mma_brdf_layer1(one, D_t, X_t, W_s + OFFB_BW1); })) break;
     epilogue_hidden(D_w, H_w);
-    if (!run_mma([&] { mma_layer2(D_t, H_t, W_s + OFFB_BW2, W_s + OFFB_ONES, W_s + OFFB_BB2); })) break;
+    if (!run_mma([&](uint32_t one) { mma_layer2(one, D_t, H_t, W_s + OFFB_BW2, W_s + OFFB_ONES, W_s + OFFB_BB2); })) break;
     {
       float dy[7];
       const float dnn = dot(n2, dn2);
@@ -608,10 +611,10 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
     // primary I backward: forward recomputed in split precision, back-propagated in bf16 (layer-1
     // input and hidden layer taken as their hi parts)
     store_primary_split(fpix, ps, X_w, H_w, wi);
-    if (!run_mma([&] { mma_layer1_split(D_t, X_t, H_t, W_s + OFFB_IW1, W_s + OFFB_IW1L); })) break;
+    if (!run_mma([&](uint32_t one) { mma_layer1_split(one, D_t, X_t, H_t, W_s + OFFB_IW1, W_s + OFFB_IW1L); })) break;
     epilogue_hidden_split(D_w, H_w, X_w);   // hi parts into H (layer 2's input as layer_backward reads it), lo into X
-    if (!run_mma([&] {
-          mma_layer2_split(D_t, H_t, X_t, W_s + OFFB_IW2, W_s + OFFB_IW2L, W_s + OFFB_ONES, W_s + OFFB_IB2);
+    if (!run_mma([&](uint32_t one) {
+          mma_layer2_split(one, D_t, H_t, X_t, W_s + OFFB_IW2, W_s + OFFB_IW2L, W_s + OFFB_ONES, W_s + OFFB_IB2);
         }))
       break;
     store_primary_hi(fpix, ps, X_w, wi);   // the layer-1 input's hi parts back into X

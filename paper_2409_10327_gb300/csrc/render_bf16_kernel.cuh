@@ -96,7 +96,8 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x;
-  const int wg = tid >> 7, t = tid & 127, warp = t >> 5, lane = t & 31;
+  const int wg = __shfl_sync(0xffffffffu, tid >> 7, 0), t = tid & 127, lane = t & 31;
+  const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);   // warp-uniform, as is what the MMA issue takes
   uint8_t* Wsm = sm + SM_W;
   uint8_t* wgb = sm + SM_WG + wg * L::kWgBytes;
   uint8_t* fpix = wgb + WG_FPIX;
@@ -122,7 +123,7 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot + (uint32_t)(128 * wg);
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0) + (uint32_t)(128 * wg);
   const uint32_t D_t = tmem + TM_D, X_t = tmem + TM_X, H_t = tmem + TM_H;   // MMA operands (lane 0)
   const uint32_t lane_off = (uint32_t)(32 * warp) << 16;                    // this warp's 32 lanes
   const uint32_t D_w = D_t + lane_off, X_w = X_t + lane_off, H_w = H_t + lane_off;
@@ -154,10 +155,12 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
     tc_fence_before();
     abort = wg_sync_or(wg, abort);
     if (abort) return false;
-    if (t == 0) {
+    if (warp == 0) {
+      const uint32_t one = elect_one();
       tc_fence_after();
-      issue();
-      mma_commit(bar_a);
+      issue(one);
+      mma_commit(one, bar_a);
+      __syncwarp();
     }
     if (!mbar_wait(bar_a, phase)) {
       if (!abort && t == 0) atomicOr(m.status, kStatusTimeout | 1u);
@@ -240,9 +243,9 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
       // (d) x' = x + t w_i and f' = H(x'); (b) B(f')
       encode_point_tmem(m.grid, x + wi * qw.w, X_w);
       store_bias_cols_tmem(X_w);
-      if (!run_mma([&] { mma_brdf_layer1(D_t, X_t, W_s + OFFB_BW1); })) return false;
+      if (!run_mma([&](uint32_t one) { mma_brdf_layer1(one, D_t, X_t, W_s + OFFB_BW1); })) return false;
       epilogue_hidden(D_w, H_w);
-      if (!run_mma([&] { mma_layer2(D_t, H_t, W_s + OFFB_BW2, W_s + OFFB_ONES, W_s + OFFB_BB2); })) return false;
+      if (!run_mma([&](uint32_t one) { mma_layer2(one, D_t, H_t, W_s + OFFB_BW2, W_s + OFFB_ONES, W_s + OFFB_BB2); })) return false;
       f3 n2, a2;
       float r2;
       {
@@ -266,9 +269,9 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
         f3 lej = mk(0.f, 0.f, 0.f);
         if (NL == 1) lej = env_fetch(envs, tapj);
         store_pe_tmem(X_w, wj);
-        if (!run_mma([&] { mma_layer1(D_t, X_t, W_s + OFFB_IW1); })) return false;
+        if (!run_mma([&](uint32_t one) { mma_layer1(one, D_t, X_t, W_s + OFFB_IW1); })) return false;
         epilogue_hidden(D_w, H_w);
-        if (!run_mma([&] { mma_layer2(D_t, H_t, W_s + OFFB_IW2, W_s + OFFB_ONES, W_s + OFFB_IB2); })) return false;
+        if (!run_mma([&](uint32_t one) { mma_layer2(one, D_t, H_t, W_s + OFFB_IW2, W_s + OFFB_ONES, W_s + OFFB_IB2); })) return false;
         const float v2 = visibility_from_logit(head_vis(D_w, hp.iw3v, hp.ib3[0]), m.force_vis2, 1);
         const f3 wj3 = frw * (wsec * v2);
         if (NL == 1) {
@@ -311,10 +314,10 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
       store_primary_split(fpix, ps, X_w, H_w, wi);
 
       // (c) I(f, w_i) in split precision: the hit test and the depth
-      if (!run_mma([&] { mma_layer1_split(D_t, X_t, H_t, W_s + OFFB_IW1, W_s + OFFB_IW1L); })) { ok = false; break; }
+      if (!run_mma([&](uint32_t one) { mma_layer1_split(one, D_t, X_t, H_t, W_s + OFFB_IW1, W_s + OFFB_IW1L); })) { ok = false; break; }
       epilogue_hidden_split(D_w, X_w, H_w);
-      if (!run_mma([&] {
-            mma_layer2_split(D_t, X_t, H_t, W_s + OFFB_IW2, W_s + OFFB_IW2L, W_s + OFFB_ONES, W_s + OFFB_IB2);
+      if (!run_mma([&](uint32_t one) {
+            mma_layer2_split(one, D_t, X_t, H_t, W_s + OFFB_IW2, W_s + OFFB_IW2L, W_s + OFFB_ONES, W_s + OFFB_IB2);
           })) {
         ok = false;
         break;
@@ -445,10 +448,10 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
       store_primary_split(fpix, ps, X_w, H_w, wi);
 
       // (c) I(f, w_i) in split precision: it alone sets t, and so x'
-      if (!run_mma([&] { mma_layer1_split(D_t, X_t, H_t, W_s + OFFB_IW1, W_s + OFFB_IW1L); })) break;
+      if (!run_mma([&](uint32_t one) { mma_layer1_split(one, D_t, X_t, H_t, W_s + OFFB_IW1, W_s + OFFB_IW1L); })) break;
       epilogue_hidden_split(D_w, X_w, H_w);
-      if (!run_mma([&] {
-            mma_layer2_split(D_t, X_t, H_t, W_s + OFFB_IW2, W_s + OFFB_IW2L, W_s + OFFB_ONES, W_s + OFFB_IB2);
+      if (!run_mma([&](uint32_t one) {
+            mma_layer2_split(one, D_t, X_t, H_t, W_s + OFFB_IW2, W_s + OFFB_IW2L, W_s + OFFB_ONES, W_s + OFFB_IB2);
           }))
         break;
       float v, tdep;
@@ -494,9 +497,9 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
       store_bias_cols_tmem(X_w);
 
       // (b) B(f')
-      if (!run_mma([&] { mma_brdf_layer1(D_t, X_t, W_s + OFFB_BW1); })) break;
+      if (!run_mma([&](uint32_t one) { mma_brdf_layer1(one, D_t, X_t, W_s + OFFB_BW1); })) break;
       epilogue_hidden(D_w, H_w);
-      if (!run_mma([&] { mma_layer2(D_t, H_t, W_s + OFFB_BW2, W_s + OFFB_ONES, W_s + OFFB_BB2); })) break;
+      if (!run_mma([&](uint32_t one) { mma_layer2(one, D_t, H_t, W_s + OFFB_BW2, W_s + OFFB_ONES, W_s + OFFB_BB2); })) break;
       f3 n2, a2;
       float r2;
       {
@@ -521,10 +524,10 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
         f3 lej = mk(0.f, 0.f, 0.f);
         if (NL == 1) lej = env_fetch(envs, tapj);
         store_pe_tmem(X_w, wj);
-        ok = run_mma([&] { mma_layer1(D_t, X_t, W_s + OFFB_IW1); });
+        ok = run_mma([&](uint32_t one) { mma_layer1(one, D_t, X_t, W_s + OFFB_IW1); });
         if (!ok) break;
         epilogue_hidden(D_w, H_w);
-        ok = run_mma([&] { mma_layer2(D_t, H_t, W_s + OFFB_IW2, W_s + OFFB_ONES, W_s + OFFB_IB2); });
+        ok = run_mma([&](uint32_t one) { mma_layer2(one, D_t, H_t, W_s + OFFB_IW2, W_s + OFFB_ONES, W_s + OFFB_IB2); });
         if (!ok) break;
         const float v2 = m.force_vis2 >= 0.f ? m.force_vis2 : sigmoid_fast(head_vis(D_w, hp.iw3v, hp.ib3[0]));
         const f3 wj3 = frw * (own ? wsec * v2 : 0.0f);

@@ -207,7 +207,7 @@ render_fp32_kernel(const __grid_constant__ ModelDesc m, rt_gbuffer gb, int P, lo
       const uint32_t one = elect_one();
       tc_fence_after();
       chain(one);
-      mma_commit_one(one, bar);
+      mma_commit(one, bar);
       __syncwarp();
     }
     return true;

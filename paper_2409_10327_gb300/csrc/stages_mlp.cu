@@ -93,7 +93,7 @@ mlp_rows_kernel(const __grid_constant__ ModelDesc m, const float* __restrict__ f
       const uint32_t one = elect_one();
       tc_fence_after();
       chain(one);
-      mma_commit_one(one, bar);
+      mma_commit(one, bar);
       __syncwarp();
     }
     return true;

@@ -47,26 +47,40 @@ __device__ __forceinline__ uint64_t sdesc32(uint32_t saddr) {
   return d;
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+// Issue.  A whole warp runs a chain's code with one lane elected (`one`, a
+// predicate of each instruction): in a one-thread branch every operand has to
+// be moved to uniform registers first, which for short MMAs (32 cycles each)
+// takes longer than the MMA.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void mma_bf16(uint32_t one, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accum) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum), "r"(one)
       : "memory");
 }
 // The same with the A operand in tensor memory (rows in lanes, K-major bf16 pairs).
-__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
-                                            uint32_t accum) {
+__device__ __forceinline__ void mma_bf16_ts(uint32_t one, uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,
+                                            uint32_t idesc, uint32_t accum) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accum)
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accum), "r"(one)
       : "memory");
 }
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
+// (by the lane that issued the chain)
+__device__ __forceinline__ void mma_commit(uint32_t one, uint32_t bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
+      "r"(one)
+      : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -143,21 +157,21 @@ __device__ __forceinline__ uint32_t pack_residual(float a, float b, uint32_t hi)
 }
 
 // D <- X . W1^T (k-steps 0..3 of the layer-1 input in TMEM)
-__device__ __forceinline__ void mma_layer1(uint32_t d, uint32_t x_t, uint32_t w_s) {
+__device__ __forceinline__ void mma_layer1(uint32_t one, uint32_t d, uint32_t x_t, uint32_t w_s) {
 #pragma unroll
-  for (int k = 0; k < 4; ++k) mma_bf16_ts(d, x_t + 8 * k, sdesc(w_s + 32 * k), kIdescN64, k > 0 ? 1u : 0u);
+  for (int k = 0; k < 4; ++k) mma_bf16_ts(one, d, x_t + 8 * k, sdesc(w_s + 32 * k), kIdescN64, k > 0 ? 1u : 0u);
 }
 // layer 2: D <- H . W2^T + ones . Bias2^T
-__device__ __forceinline__ void mma_layer2(uint32_t d, uint32_t h_t, uint32_t w_s, uint32_t ones_s, uint32_t bias_s) {
+__device__ __forceinline__ void mma_layer2(uint32_t one, uint32_t d, uint32_t h_t, uint32_t w_s, uint32_t ones_s, uint32_t bias_s) {
 #pragma unroll
-  for (int k = 0; k < 4; ++k) mma_bf16_ts(d, h_t + 8 * k, sdesc(w_s + 32 * k), kIdescN64, k > 0 ? 1u : 0u);
-  mma_bf16(d, sdesc32(ones_s), sdesc32(bias_s), kIdescN64, 1u);
+  for (int k = 0; k < 4; ++k) mma_bf16_ts(one, d, h_t + 8 * k, sdesc(w_s + 32 * k), kIdescN64, k > 0 ? 1u : 0u);
+  mma_bf16(one, d, sdesc32(ones_s), sdesc32(bias_s), kIdescN64, 1u);
 }
 // B's layer 1: f' (k-steps 0, 1) and the bias columns (k-step 3; B's weights are zero on the PE columns)
-__device__ __forceinline__ void mma_brdf_layer1(uint32_t d, uint32_t x_t, uint32_t w_s) {
-  mma_bf16_ts(d, x_t, sdesc(w_s), kIdescN64, 0u);
-  mma_bf16_ts(d, x_t + 8, sdesc(w_s + 32), kIdescN64, 1u);
-  mma_bf16_ts(d, x_t + 24, sdesc(w_s + 96), kIdescN64, 1u);
+__device__ __forceinline__ void mma_brdf_layer1(uint32_t one, uint32_t d, uint32_t x_t, uint32_t w_s) {
+  mma_bf16_ts(one, d, x_t, sdesc(w_s), kIdescN64, 0u);
+  mma_bf16_ts(one, d, x_t + 8, sdesc(w_s + 32), kIdescN64, 1u);
+  mma_bf16_ts(one, d, x_t + 24, sdesc(w_s + 96), kIdescN64, 1u);
 }
 
 // The primary evaluation of I in split precision.  Every operand is a bf16
@@ -167,20 +181,20 @@ __device__ __forceinline__ void mma_brdf_layer1(uint32_t d, uint32_t x_t, uint32
 // during layer 1 (and X / H hold the hi / lo parts of the hidden layer during
 // layer 2), so the warpgroup's 128 TMEM columns suffice.
 // Layer 1: D <- Xh W1h + Xl W1h + Xh W1l (the bias rides on Xh's ones columns).
-__device__ __forceinline__ void mma_layer1_split(uint32_t d, uint32_t xh_t, uint32_t xl_t, uint32_t w_s,
+__device__ __forceinline__ void mma_layer1_split(uint32_t one, uint32_t d, uint32_t xh_t, uint32_t xl_t, uint32_t w_s,
                                                  uint32_t wl_s) {
 #pragma unroll
-  for (int k = 0; k < 4; ++k) mma_bf16_ts(d, xh_t + 8 * k, sdesc(w_s + 32 * k), kIdescN64, k > 0 ? 1u : 0u);
+  for (int k = 0; k < 4; ++k) mma_bf16_ts(one, d, xh_t + 8 * k, sdesc(w_s + 32 * k), kIdescN64, k > 0 ? 1u : 0u);
 #pragma unroll
-  for (int k = 0; k < 4; ++k) mma_bf16_ts(d, xl_t + 8 * k, sdesc(w_s + 32 * k), kIdescN64, 1u);
+  for (int k = 0; k < 4; ++k) mma_bf16_ts(one, d, xl_t + 8 * k, sdesc(w_s + 32 * k), kIdescN64, 1u);
 #pragma unroll
-  for (int k = 0; k < 4; ++k) mma_bf16_ts(d, xh_t + 8 * k, sdesc(wl_s + 32 * k), kIdescN64, 1u);
+  for (int k = 0; k < 4; ++k) mma_bf16_ts(one, d, xh_t + 8 * k, sdesc(wl_s + 32 * k), kIdescN64, 1u);
 }
 // Layer 2: D <- Hh W2h + Hl W2h + Hh W2l + ones . Bias2
-__device__ __forceinline__ void mma_layer2_split(uint32_t d, uint32_t hh_t, uint32_t hl_t, uint32_t w_s,
+__device__ __forceinline__ void mma_layer2_split(uint32_t one, uint32_t d, uint32_t hh_t, uint32_t hl_t, uint32_t w_s,
                                                  uint32_t wl_s, uint32_t ones_s, uint32_t bias_s) {
-  mma_layer1_split(d, hh_t, hl_t, w_s, wl_s);
-  mma_bf16(d, sdesc32(ones_s), sdesc32(bias_s), kIdescN64, 1u);
+  mma_layer1_split(one, d, hh_t, hl_t, w_s, wl_s);
+  mma_bf16(one, d, sdesc32(ones_s), sdesc32(bias_s), kIdescN64, 1u);
 }
 // Split hidden epilogue: Hh = bf16(relu(D)), Hl = bf16(relu(D) - Hh), 16 columns at a time.
 __device__ __forceinline__ void epilogue_hidden_split(uint32_t d_taddr, uint32_t hh_taddr, uint32_t hl_taddr) {

@@ -103,41 +103,10 @@ __device__ __forceinline__ void build_heads(float* hd, const float* __restrict__
 // The layer-1 tile of I takes [f (32) | PE (32)]: the feature and PE rows of the packed image are adjacent.
 static_assert(OFF_IW1P == OFF_IW1F + 32 * 64, "I's layer 1 is one [64][64] block");
 
-// A chain is up to 49 MMAs of 32 cycles, so their issue must not cost more than
-// that: one whole warp runs the chain's code with one lane elected (`one`, by
-// predicate) instead of one thread in a divergent branch, which keeps the
-// operands in uniform registers.
-__device__ __forceinline__ uint32_t elect_one() {
-  uint32_t r;
-  asm volatile(
-      "{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void mma_ts_one(uint32_t one, uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t accum) {
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
-      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(bdesc), "r"(kIdescN64), "r"(accum), "r"(one)
-      : "memory");
-}
-__device__ __forceinline__ void mma_ss_one(uint32_t one, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t accum) {
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
-      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(kIdescN64), "r"(accum), "r"(one)
-      : "memory");
-}
-__device__ __forceinline__ void mma_commit_one(uint32_t one, uint32_t bar) {
-  asm volatile(
-      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
-      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
-      "r"(one)
-      : "memory");
-}
 template <int K0, int K1>
 __device__ __forceinline__ void mma_part(uint32_t one, uint32_t d, uint32_t a_t, uint32_t w_s, uint32_t first) {
 #pragma unroll
-  for (int k = K0; k < K1; ++k) mma_ts_one(one, d, a_t + 8 * k, sdesc(w_s + 32 * k), (k > K0 || !first) ? 1u : 0u);
+  for (int k = K0; k < K1; ++k) mma_bf16_ts(one, d, a_t + 8 * k, sdesc(w_s + 32 * k), kIdescN64, (k > K0 || !first) ? 1u : 0u);
 }
 // D <- A W^T over the input columns [16 K0, 16 K1); a: part 0 in TMEM (parts 32 columns apart), w: part 0 in shared memory.
 template <int K0, int K1>
@@ -152,7 +121,7 @@ __device__ __forceinline__ void mma_split3(uint32_t one, uint32_t d, uint32_t a,
 // Layer 2: D <- ones Bias2^T + A W^T (the bias first, like the FP32 sums it replaces)
 __device__ __forceinline__ void mma_split3_layer2(uint32_t one, uint32_t d, uint32_t a, uint32_t w, uint32_t ones,
                                                   uint32_t bias) {
-  mma_ss_one(one, d, sdesc32(ones), sdesc32(bias), 0u);
+  mma_bf16(one, d, sdesc32(ones), sdesc32(bias), kIdescN64, 0u);
   mma_split3<0, 4>(one, d, a, w, 0u);
 }
 // B's layer 1: the features, and part 0 of the ones columns (its weights are zero on the PE columns)
