@@ -11,13 +11,15 @@
 // few MB at 800 x 800 and stays in L2 across the passes; taps hit L1.  The
 // kernels are bound by instruction issue, so a tap is kept short:
 //   - the edge-stopping functions multiply to one power of two, w = 2^-(a_z +
-//     a_l + sigma_n L) in units of log2(e), L = -ln(n . n') (neg_ln below);
+//     a_l + sigma_n L) in units of log2(e), L = -ln(n . n') (edge_weights below);
 //   - the depth term's divisor depends on the offset alone and is equal for
 //     opposite offsets: 12 (24 in the 7 x 7 window) reciprocals per pixel
 //     instead of 25 (49) divisions;
 //   - blocks whose whole window lies inside the image address taps by
-//     constant offsets from one row pointer, without bounds tests.
-// 800 x 800, five passes: 270 us; with expf twice, powf and a division per
+//     constant offsets from one row pointer, without bounds tests;
+//   - a window row's taps are loaded before any is weighted, and share one
+//     test for the logarithm's series (270 us with a test per tap).
+// 800 x 800, five passes: 229 us; with expf twice, powf and a division per
 // tap 596 us (error against 64 bits 2.7e-7 both).
 #include "device_common.cuh"
 
@@ -26,6 +28,7 @@ namespace {
 
 constexpr float kEps = 1e-10f;
 constexpr float kLog2e = 1.44269504088896340736f;
+constexpr float kOutside = 1e30f;   // the exponent of a tap outside the image: weight 0
 constexpr int kBX = 32, kBY = 8;
 
 __device__ __forceinline__ float luminance(float4 c) { return 0.2126f * c.x + 0.7152f * c.y + 0.0722f * c.z; }
@@ -39,33 +42,39 @@ __device__ __forceinline__ float2 depth_gradient(const float* __restrict__ z, in
   return make_float2(gx, gy);
 }
 
-// -ln(c) for c = n . n': with d = 1 - c (exact for c in [1/2, 2]) the series
-// d + d^2/2 + ... + d^9/9 where |d| < 1/8 (its remainder is below 2^-28 of the
-// sum), which neighbouring taps of a smooth surface take; the library
-// logarithm elsewhere (a normal edge).
-__device__ __forceinline__ float neg_ln(float c) {
-  const float d = 1.0f - c;
-  if (fabsf(d) < 0.125f) {
-    float s = 1.0f / 9.0f;
-    s = fmaf(s, d, 1.0f / 8.0f);
-    s = fmaf(s, d, 1.0f / 7.0f);
-    s = fmaf(s, d, 1.0f / 6.0f);
-    s = fmaf(s, d, 1.0f / 5.0f);
-    s = fmaf(s, d, 1.0f / 4.0f);
-    s = fmaf(s, d, 1.0f / 3.0f);
-    s = fmaf(s, d, 0.5f);
-    return fmaf(s * d, d, d);
-  }
-  return -logf(fmaxf(c, 0.0f));   // c <= 0: +inf, weight 0
+// -ln(c) for c = n . n' by the series of d = 1 - c (exact for c in [1/2, 2]), d + d^2/2 + ... + d^9/9.  For |d| < 1/8,
+// which neighbouring taps of a smooth surface have, the remainder is below 2^-28 of the sum.
+__device__ __forceinline__ float neg_ln_series(float d) {
+  float s = 1.0f / 9.0f;
+  s = fmaf(s, d, 1.0f / 8.0f);
+  s = fmaf(s, d, 1.0f / 7.0f);
+  s = fmaf(s, d, 1.0f / 6.0f);
+  s = fmaf(s, d, 1.0f / 5.0f);
+  s = fmaf(s, d, 1.0f / 4.0f);
+  s = fmaf(s, d, 1.0f / 3.0f);
+  s = fmaf(s, d, 0.5f);
+  return fmaf(s * d, d, d);
 }
 
-// w_z w_n w_l of a tap as one power of two: a is log2(e) times the depth and luminance exponent (>= 0), c = n . n',
-// sn = sigma_n log2(e); NORMAL: sigma_n > 0
-template <bool NORMAL>
-__device__ __forceinline__ float edge_weight(float a, float c, float sn) {
-  float w;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(-(NORMAL ? fmaf(sn, neg_ln(c), a) : a)));   // max(0, c)^0 = 1
-  return w;
+// Weights w_z w_n w_l of a row of D taps, each one power of two: a[k] is log2(e) times the depth and luminance exponent
+// (>= 0), c[k] = n . n', sn = sigma_n log2(e); NORMAL: sigma_n > 0.  The row takes the series as a whole (one test per
+// row and no divergence on smooth surfaces), or the library logarithm (a normal edge; c <= 0 or NaN: weight 0).
+template <bool NORMAL, int D>
+__device__ __forceinline__ void edge_weights(float (&a)[D], const float (&c)[D], float sn, float (&w)[D]) {
+  if constexpr (NORMAL) {
+    bool near = true;
+#pragma unroll
+    for (int k = 0; k < D; ++k) near = near && fabsf(1.0f - c[k]) < 0.125f;
+    if (near) {
+#pragma unroll
+      for (int k = 0; k < D; ++k) a[k] = fmaf(sn, neg_ln_series(1.0f - c[k]), a[k]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < D; ++k) a[k] = fmaf(sn, -logf(fmaxf(c[k], 0.0f)), a[k]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < D; ++k) asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(w[k]) : "f"(-a[k]));   // max(0, c)^0 = 1
 }
 
 // The depth term's divisors as factors, log2(e) / (sigma_z |g . s| + eps), for the
@@ -98,16 +107,26 @@ __device__ __forceinline__ void variance_pixel(int W, int H, int x, int y, const
     const int qy = y + dy;
     if (!INTERIOR && (qy < 0 || qy >= H)) continue;
     const int row = p + dy * W;
+    float a[7], c[7], w[7], l[7];
 #pragma unroll
-    for (int dx = -3; dx <= 3; ++dx) {
-      if (!INTERIOR && (x + dx < 0 || x + dx >= W)) continue;
-      const int q = row + dx;
-      const float a = fabsf(zp - __ldg(z + q)) * inv[(dy + 3) * 7 + dx + 3];
-      const float w = edge_weight<NORMAL>(a, dot(np_, xyz(__ldg(nrm + q))), sn);
-      const float l = luminance(__ldg(rad + q));
-      s0 += w;
-      s1 += w * l;
-      s2 += w * l * l;
+    for (int k = 0; k < 7; ++k) {
+      const bool in = INTERIOR || (x + k - 3 >= 0 && x + k - 3 < W);
+      a[k] = kOutside;
+      c[k] = 1.0f;
+      l[k] = 0.0f;
+      if (in) {
+        const int q = row + k - 3;
+        a[k] = fabsf(zp - __ldg(z + q)) * inv[(dy + 3) * 7 + k];
+        c[k] = dot(np_, xyz(__ldg(nrm + q)));
+        l[k] = luminance(__ldg(rad + q));
+      }
+    }
+    edge_weights<NORMAL>(a, c, sn, w);
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+      s0 += w[k];
+      s1 += w[k] * l[k];
+      s2 += w[k] * l[k] * l[k];
     }
   }
   const float m1 = s1 / s0, m2 = s2 / s0;
@@ -116,7 +135,7 @@ __device__ __forceinline__ void variance_pixel(int W, int H, int x, int y, const
 }
 
 template <bool NORMAL>
-__global__ void __launch_bounds__(kBX* kBY)
+__global__ void __launch_bounds__(kBX* kBY, 3)
 svgf_variance_kernel(int W, int H, const float4* __restrict__ rad, const float* __restrict__ z,
                      const float4* __restrict__ nrm, float sigma_z, float sigma_n, float4* __restrict__ out) {
   const int gx = (W + kBX - 1) / kBX;   // blocks in row order on one grid axis: no limit on the height
@@ -161,19 +180,31 @@ __device__ __forceinline__ void atrous_pixel(int W, int H, int step, int x, int 
     const int qy = y + step * dy;
     if (!INTERIOR && (qy < 0 || qy >= H)) continue;
     const int row = p + step * dy * W;
+    float4 cq[5];
+    float a[5], c[5], w[5];
 #pragma unroll
-    for (int dx = -2; dx <= 2; ++dx) {
-      const int qx = x + step * dx;
-      if (!INTERIOR && (qx < 0 || qx >= W)) continue;
-      const int q = row + step * dx;
-      const float4 cq = __ldg(in + q);
-      const float a = fmaf(fabsf(lp - luminance(cq)), inv_l, fabsf(zp - __ldg(z + q)) * inv[(dy + 2) * 5 + dx + 2]);
-      const float w = h1[dy + 2] * h1[dx + 2] * edge_weight<NORMAL>(a, dot(np_, xyz(__ldg(nrm + q))), sn);
-      ws += w;
-      ax += w * cq.x;
-      ay += w * cq.y;
-      az += w * cq.z;
-      av += w * w * cq.w;
+    for (int k = 0; k < 5; ++k) {
+      const int qx = x + step * (k - 2);
+      const bool in_x = INTERIOR || (qx >= 0 && qx < W);
+      a[k] = kOutside;
+      c[k] = 1.0f;
+      cq[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (in_x) {
+        const int q = row + step * (k - 2);
+        cq[k] = __ldg(in + q);
+        a[k] = fmaf(fabsf(lp - luminance(cq[k])), inv_l, fabsf(zp - __ldg(z + q)) * inv[(dy + 2) * 5 + k]);
+        c[k] = dot(np_, xyz(__ldg(nrm + q)));
+      }
+    }
+    edge_weights<NORMAL>(a, c, sn, w);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      const float wk = h1[dy + 2] * h1[k] * w[k];
+      ws += wk;
+      ax += wk * cq[k].x;
+      ay += wk * cq[k].y;
+      az += wk * cq[k].z;
+      av += wk * wk * cq[k].w;
     }
   }
   const float inv_w = 1.0f / ws;
@@ -181,7 +212,7 @@ __device__ __forceinline__ void atrous_pixel(int W, int H, int step, int x, int 
 }
 
 template <bool NORMAL>
-__global__ void __launch_bounds__(kBX* kBY)
+__global__ void __launch_bounds__(kBX* kBY, 3)
 svgf_atrous_kernel(int W, int H, int step, const float4* __restrict__ in, const float* __restrict__ z,
                    const float4* __restrict__ nrm, float sigma_z, float sigma_n, float sigma_l,
                    float4* __restrict__ out) {
