@@ -2,24 +2,26 @@
 // given features and directions (rt_trace; also the distillation's teacher).
 // Rows, (point) or (point, direction) consecutively, run 128 at a time through
 // the tensor-core layers of tc_split.cuh, as in the FP32 frame kernel: a
-// warpgroup per tile, thread = row = TMEM lane, two warpgroups per SM that
-// take turns on the tensor pipe.  Within a warpgroup the next tile's input is
-// made while layer 2 of the current one runs (layer 1 has read it by then).
-// A tile is 49 MMAs of 32 cycles against about 1,000 instructions per warp.
+// warpgroup per tile, thread = row = TMEM lane, three warpgroups per SM that
+// take turns on the tensor pipe.  Within a warpgroup the next tile's features
+// and encoding are made while layer 2 of the current one runs.
+// A tile is 49 MMAs of 32 cycles against about 1,000 instructions per warp and
+// waits on its chains and TMEM reads, hence as many warpgroups as tensor memory
+// holds: 160 columns each, the hidden operand taking the input's columns (two
+// of 256 columns: 169 us for the trace below).
 // 100,003 points with 16 directions: rt_encode + rt_decode + rt_trace took
 // 1,184 us with a warp per 32 directions of a point (half of the lanes idle at
-// 16) and a thread per decoded point; now 292 us, of it the trace 229 us and
-// the decode 36 us.
+// 16) and a thread per decoded point; now 209 us.
 #include "tc_split.cuh"
 
 namespace rtk {
 
 namespace {
 
-constexpr int kWG = 2;
+constexpr int kWG = 3;
 constexpr int kThreads = 128 * kWG;
-constexpr int kTmemCols = 256 * kWG;
-constexpr int TM_D = 0, TM_X = 64, TM_H = 160;   // as in render_fp32.cu
+constexpr int kTmemCols = 512;   // 160 per warpgroup; allocations are powers of two
+constexpr int TM_D = 0, TM_X = 64, TM_H = TM_X;   // H takes X's columns once layer 1 has read them
 // shared memory: one MLP's split weights and output layers, then per warpgroup the tile's split features and a barrier
 constexpr int SM_W1 = 0, SM_W2 = 3 * kPart, SM_B2 = 6 * kPart, SM_ONES = SM_B2 + 2048, SM_HEAD = SM_ONES + 4096;
 constexpr int SM_WG = SM_HEAD + HD_FLOATS * 4;
@@ -74,7 +76,7 @@ mlp_rows_kernel(const __grid_constant__ ModelDesc m, const float* __restrict__ f
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0) + (uint32_t)(256 * wg);
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0) + (uint32_t)(160 * wg);
   const uint32_t D_t = tmem + TM_D, X_t = tmem + TM_X, H_t = tmem + TM_H;
   const uint32_t lane_off = (uint32_t)(32 * warp) << 16;
   const uint32_t D_w = D_t + lane_off, X_w = X_t + lane_off, H_w = H_t + lane_off;
@@ -108,14 +110,13 @@ mlp_rows_kernel(const __grid_constant__ ModelDesc m, const float* __restrict__ f
     tc_fence_after();
   };
 
-  // The split layer-1 input of the tile's rows: features through shared memory
-  // (split once per point) where the tile spans few points, else per row.
-  auto load_tile = [&](long long tile) {
+  // The split layer-1 input of a tile's rows: features through shared memory (split once per point) where the tile
+  // spans few points, else per row when they are stored; the encoding in registers.
+  uint32_t pe0[16], pe1[16], pe2[16];
+  auto prepare_tile = [&](long long tile) {
     const long long r0 = tile * 128, r1 = min(r0 + 128, rows) - 1;
     const long long p0 = r0 / K;
     const int np = (int)(r1 / K - p0) + 1;
-    const long long r = min(r0 + t, r1);
-    const long long p = r / K;
     wg_sync(wg);   // the previous tile's slots are read
     if (np <= kPixSlots) {
       for (int e = t; e < np * 16; e += 128) {
@@ -127,7 +128,16 @@ mlp_rows_kernel(const __grid_constant__ ModelDesc m, const float* __restrict__ f
         d[16] = q1;
         d[32] = q2;
       }
-      wg_sync(wg);
+    }
+    // B reads the ones columns only: its weights are zero on the encoding's
+    pe_split3(IRT ? xyz(__ldg(dirs + min(r0 + t, r1))) : mk(0.f, 0.f, 0.f), pe0, pe1, pe2);
+    wg_sync(wg);
+  };
+  auto store_input = [&](long long tile) {
+    const long long r0 = tile * 128, r1 = min(r0 + 128, rows) - 1;
+    const long long p0 = r0 / K, p = min(r0 + t, r1) / K;
+    tmem_st16x3(X_w + 16, pe0, pe1, pe2);
+    if ((int)(r1 / K - p0) + 1 <= kPixSlots) {
       const uint8_t* src = slots + (int)(p - p0) * kSlot;
 #pragma unroll
       for (int part = 0; part < 3; ++part) {
@@ -143,7 +153,6 @@ mlp_rows_kernel(const __grid_constant__ ModelDesc m, const float* __restrict__ f
         tmem_st16(X_w + 32 * part, fr);
       }
     } else {
-      wg_sync(wg);
       uint32_t q0[16], q1[16], q2[16];
 #pragma unroll
       for (int e = 0; e < 16; ++e) {
@@ -152,14 +161,15 @@ mlp_rows_kernel(const __grid_constant__ ModelDesc m, const float* __restrict__ f
       }
       tmem_st16x3(X_w, q0, q1, q2);
     }
-    // B reads the ones columns only: its weights are zero on the encoding's
-    store_pe_split3(X_w, IRT ? xyz(__ldg(dirs + r)) : mk(0.f, 0.f, 0.f));
   };
 
   const long long ntiles = (rows + 127) / 128;
   const long long stride = (long long)gridDim.x * kWG;
   long long tile = (long long)blockIdx.x * kWG + wg;
-  if (tile < ntiles) load_tile(tile);
+  if (tile < ntiles) {
+    prepare_tile(tile);
+    store_input(tile);
+  }
   for (; tile < ntiles; tile += stride) {
     if (!issue([&](uint32_t one) {
           if (IRT) mma_split3<0, 4>(one, D_t, X_t, S + SM_W1);
@@ -169,8 +179,9 @@ mlp_rows_kernel(const __grid_constant__ ModelDesc m, const float* __restrict__ f
     wait();
     epilogue_split3(D_w, H_w);
     if (!issue([&](uint32_t one) { mma_split3_layer2(one, D_t, H_t, S + SM_W2, S + SM_ONES, S + SM_B2); })) break;
-    if (tile + stride < ntiles) load_tile(tile + stride);
+    if (tile + stride < ntiles) prepare_tile(tile + stride);
     wait();
+    if (tile + stride < ntiles) store_input(tile + stride);
     const long long r = tile * 128 + t;
     if (IRT) {
       float z[2];
