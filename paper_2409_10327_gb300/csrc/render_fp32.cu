@@ -17,9 +17,9 @@
 // computes, and within a warpgroup the BRDF and environment lookup of a
 // direction overlap its layer 1, and the next direction and its encoding
 // overlap its layer 2.
-// 800 x 800 x 128 directions: 166 ms, 247 ms with every evaluation on the FMA
+// 800 x 800 x 128 directions: 133 ms, 247 ms with every evaluation on the FMA
 // pipes; 97 x 61 x 40 (consecutive rows instead of 32 directions of one pixel
-// per warp, which wasted three rows in eight there): 515 us, 1,164 us.
+// per warp, which wasted three rows in eight there): 422 us, 1,164 us.
 //
 // TMEM columns of a warpgroup (256 from column 256 * wg):
 //   D [0, 64)     FP32 accumulator of both layers
@@ -42,15 +42,16 @@ constexpr int kWG = 2;
 constexpr int kThreads = 128 * kWG;
 constexpr int kTmemCols = 256 * kWG;
 constexpr int TM_D = 0, TM_X = 64, TM_H = 160;
+constexpr int kSlots = 10;       // pixels of a tile whose feature part of layer 1 is shared (N >= 16)
 // shared memory from a 1024-aligned base: I's split weights (parts, layer-2 bias, ones), the packed FP32 image, I's
 // visibility row, an activation buffer per warp, then per warpgroup
 constexpr int SM_W1 = 0, SM_W2 = 3 * kPart, SM_B2 = 6 * kPart, SM_ONES = SM_B2 + 2048;
-constexpr int SM_W = SM_ONES + 4096;                  // float [WPACK_FLOATS]
-constexpr int SM_HV = SM_W + WPACK_FLOATS * 4;        // float [64]
+constexpr int SM_W = SM_ONES + 4096;                  // float [WPACK_FLOATS - OFF_IW1P]: the packed image from I's PE rows on
+constexpr int SM_HV = SM_W + (WPACK_FLOATS - OFF_IW1P) * 4;        // float [64]
 constexpr int SM_ACT = SM_HV + 64 * 4;                // float [8 warps][kActStride]
 constexpr int SM_WG = SM_ACT + 4 * kWG * kActStride * 4;
-constexpr int WG_AP = 0;                              // float [kPixSlots][64]: b1 + W1f f of the tile's pixels
-constexpr int WG_RED = WG_AP + kPixSlots * 64 * 4;    // float4 [128]: the tile's contributions
+constexpr int WG_AP = 0;                              // float [kSlots][64]: b1 + W1f f of the tile's pixels
+constexpr int WG_RED = WG_AP + kSlots * 64 * 4;    // float4 [128]: the tile's contributions
 constexpr int WG_CARRY = WG_RED + 128 * 16;           // float4 [2][32]: lane sums of a pixel that continues, by tile parity
 constexpr int WG_BAR = WG_CARRY + 2 * 32 * 16;        // mbarrier
 constexpr int WG_BYTES = WG_BAR + 16;
@@ -59,7 +60,9 @@ constexpr size_t kSmemBytes = kTmemSlot + 16 + 1024;
 static_assert(SM_W % 16 == 0 && SM_HV % 16 == 0 && SM_ACT % 16 == 0 && SM_WG % 16 == 0 && WG_RED % 16 == 0 &&
                   WG_BYTES % 16 == 0,
               "aligned blocks");
-static_assert(kSmemBytes <= 232448, "one CTA per SM");
+// The gathers of the x' encode live on L1: a line of it per lane and corner.  One step of the shared-memory
+// configurations below the largest leaves 60 KB of the SM for L1 instead of 28 KB: 150 -> 133 ms for the frame above.
+static_assert(kSmemBytes + 1024 <= 196 * 1024, "fits the 196 KB configuration");
 
 // Four corners of level l's cell at x (corners 4 half .. 4 half + 3) weighted and summed; a level's primary feature
 // is the sum of its two halves.
@@ -86,8 +89,8 @@ __device__ __forceinline__ float2 encode_half(const GridDesc& g, int l, int half
 
 // (a) f = H(x) of one pixel (lanes 2l and 2l + 1 take half of level l each), then I's layer-1 bias b1 + W1f f, shared
 // by the pixel's directions, into aP [64]; fP: 32 floats of the warp's scratch.
-__device__ __forceinline__ void primary_bias(const GridDesc& g, f3 x, const float* sw, int lfp, float* fP, float* aP,
-                                             int lane) {
+__device__ __forceinline__ void primary_bias(const GridDesc& g, f3 x, const float* __restrict__ wpack, int lfp,
+                                             float* fP, float* aP, int lane) {
   float2 part = make_float2(0.f, 0.f);
   if ((lane >> 1) < g.levels) part = encode_half(g, lane >> 1, lane & 1, x);
   part.x += __shfl_xor_sync(0xffffffffu, part.x, 1);
@@ -100,8 +103,9 @@ __device__ __forceinline__ void primary_bias(const GridDesc& g, f3 x, const floa
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int c = lane + 32 * h;
-    float acc = sw[OFF_IB1 + c];
-    for (int k = 0; k < lfp; ++k) acc = fmaf(fP[k], sw[OFF_IW1F + k * 64 + c], acc);
+    float acc = __ldg(wpack + OFF_IB1 + c);
+#pragma unroll 8
+    for (int k = 0; k < lfp; ++k) acc = fmaf(fP[k], __ldg(wpack + OFF_IW1F + k * 64 + c), acc);
     aP[c] = acc;
   }
   __syncwarp();
@@ -147,7 +151,7 @@ render_fp32_kernel(const __grid_constant__ ModelDesc m, rt_gbuffer gb, int P, lo
   float* aP = reinterpret_cast<float*>(wgb + WG_AP);
   float4* red = reinterpret_cast<float4*>(wgb + WG_RED);
   float4* carry = reinterpret_cast<float4*>(wgb + WG_CARRY);
-  float* sw = reinterpret_cast<float*>(sm + SM_W);
+  const float* sw = reinterpret_cast<const float*>(sm + SM_W) - OFF_IW1P;   // indexed like the packed image
   float* hv = reinterpret_cast<float*>(sm + SM_HV);
   float* act = reinterpret_cast<float*>(sm + SM_ACT) + (tid >> 5) * kActStride;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + kTmemSlot);
@@ -158,8 +162,9 @@ render_fp32_kernel(const __grid_constant__ ModelDesc m, rt_gbuffer gb, int P, lo
   build_split_matrix(sm + SM_W2, m.wpack + OFF_IW2, 64, nullptr, tid, kThreads);
   build_split_bias(sm + SM_B2, m.wpack + OFF_IB2, tid, kThreads);
   build_split_ones(sm + SM_ONES, tid, kThreads);
-  for (int i = tid; i < WPACK_FLOATS / 4; i += kThreads)
-    reinterpret_cast<float4*>(sw)[i] = __ldg(reinterpret_cast<const float4*>(m.wpack) + i);
+  static_assert(OFF_IW1P % 4 == 0, "float4 copy");
+  for (int i = tid; i < (WPACK_FLOATS - OFF_IW1P) / 4; i += kThreads)
+    reinterpret_cast<float4*>(sm + SM_W)[i] = __ldg(reinterpret_cast<const float4*>(m.wpack + OFF_IW1P) + i);
   if (tid < 64) hv[tid] = __ldg(m.wpack + OFF_IW3 + 2 * tid);
   if (t == 0) {
     mbar_init(bar, 1);
@@ -245,10 +250,10 @@ render_fp32_kernel(const __grid_constant__ ModelDesc m, rt_gbuffer gb, int P, lo
                         : cosine_direction(n, m.seed, dir_counter(q, M, 0));
 
     // (a) and (c) I(f, w_i).  The feature part of layer 1 once per pixel; per row where a tile may span more pixels
-    // than there are slots (N < 4)
+    // than there are slots (N < 16)
     Tile acc;
-    if (npix <= kPixSlots) {
-      for (int s = warp; s < npix; s += 4) primary_bias(m.grid, xyz(pos4[p_first + s]), sw, lfp, act, aP + 64 * s, lane);
+    if (npix <= kSlots) {
+      for (int s = warp; s < npix; s += 4) primary_bias(m.grid, xyz(pos4[p_first + s]), m.wpack, lfp, act, aP + 64 * s, lane);
       wg_sync(wg);
       store_pe(act, wi, lane);
       __syncwarp();
@@ -274,7 +279,7 @@ render_fp32_kernel(const __grid_constant__ ModelDesc m, rt_gbuffer gb, int P, lo
 #pragma unroll
         for (int r = 0; r < 4; ++r) bias.v[r][c] = make_float2(b, b);
       }
-      warp_gemm_k(act, sw + OFF_IW1F, bias, lfp, rg, cg);
+      warp_gemm_k(act, m.wpack + OFF_IW1F, bias, lfp, rg, cg);
       __syncwarp();
       store_pe(act, wi, lane);
       __syncwarp();
