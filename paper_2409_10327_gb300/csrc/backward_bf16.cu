@@ -318,8 +318,11 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
   //     dW1 and db1 into G.
   // Each weight-gradient block goes to the caller's blob through the warp's slice of SA (global
   // reductions); db3 by warp reductions.  w1s / w2s are the forward's weight tiles, read as W^T.
+  // Round trip 2 leaves D and, once the layer input is staged, X free: `prepare` may store the next
+  // evaluation's layer-1 input there and `ride` issue its layer 1 with the trip.
   auto layer_backward = [&](const auto& dz3, auto w3, uint32_t w2s, uint32_t w1s, bool acc_f, float* gw3,
-                            float* gb3, float* gw2, float* gb2, float* gw1, float* gb1, int ldw1, auto map1) -> bool {
+                            float* gb3, float* gw2, float* gb2, float* gw1, float* gb1, int ldw1, auto map1,
+                            auto prepare, auto ride) -> bool {
     constexpr int nout = (int)(sizeof(dz3) / sizeof(float));
     uint32_t mlo = 0, mhi = 0;   // the ReLU mask of layer 1, one bit per hidden unit
     // H1 (layer 2's input) into SB, and its mask (H1 = bf16(relu(.)) is positive or zero)
@@ -426,9 +429,11 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
 #pragma unroll
       for (int k = 0; k < 4; ++k) stage_chunk(SB, t, 4 * h + k, r[4 * k], r[4 * k + 1], r[4 * k + 2], r[4 * k + 3]);
     }
+    prepare();
     if (!run_mma([&](uint32_t one) {
           mma_input_grad(one, F_t, H_t, w1s, kIdescT32, acc_f ? 1u : 0u);
           mma_weight_grad(one, G_t, SA_s, SB_s, ONES_s);
+          ride(one);
         }))
       return false;
     // dW1 (the ones columns of the input are not mapped; db1 is column 64)
@@ -443,6 +448,9 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
     __syncwarp();
     return true;
   };
+
+  const auto nothing = [] {};
+  const auto no_ride = [](uint32_t) {};
 
   for (long long sbase = p0 * N; sbase < s_end; sbase += 128) {
     const long long p_first = sbase / N;
@@ -512,12 +520,14 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
     const f3 dli = (Gp * fr1) * sN;
     const f3 dlo2 = dli * (1.0f - v);
 
-    // secondary directions: forward, then backward, of I(f', w'_j)
+    // secondary directions: forward, then backward, of I(f', w'_j).  Layer 1 of direction j + 1 rides on
+    // the last round trip of j's backward, so a direction takes three round trips.
     f3 lo2 = mk(0.f, 0.f, 0.f), da2 = mk(0.f, 0.f, 0.f), dn2 = mk(0.f, 0.f, 0.f);
     float dr2 = 0.0f;
-    bool ok = true;
+    f3 wj = cosine_direction_fast(n2, m.seed, dir_counter(q, M, 1));
+    store_pe_tmem(X_w, wj);
+    bool ok = run_mma([&](uint32_t one) { mma_layer1(one, D_t, X_t, W_s + OFFB_IW1); });
     for (int j = 0; j < M && ok; ++j) {
-      const f3 wj = cosine_direction_fast(n2, m.seed, dir_counter(q, M, 1 + j));
       const EnvTap tapj = env_tap_fast(m.env_h, m.env_w, wj);
       const f3 le = env_fetch(m.env, tapj);
       float ds_dr = 0.0f;
@@ -525,9 +535,6 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
       const float s = disney ? spec_with_grad(r2, n2, wj, wo2, m.f0, ds_dr, ds_dn) : 0.0f;
       const f3 fr2 = mk(a2.x * kInvPi + s, a2.y * kInvPi + s, a2.z * kInvPi + s);
       const f3 ef = le * fr2;
-      store_pe_tmem(X_w, wj);
-      ok = run_mma([&](uint32_t one) { mma_layer1(one, D_t, X_t, W_s + OFFB_IW1); });
-      if (!ok) break;
       epilogue_hidden(D_w, H_w);
       ok = run_mma([&](uint32_t one) { mma_layer2(one, D_t, H_t, W_s + OFFB_IW2, W_s + OFFB_ONES, W_s + OFFB_IB2); });
       if (!ok) break;
@@ -543,7 +550,17 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
         dn2 = dn2 + ds_dn * dsum;
       }
       const float dz3[1] = {m.force_vis2 >= 0.f ? 0.0f : dv2 * v2 * (1.0f - v2)};
-      ok = layer_backward(dz3, w3_i, W_s + OFFB_IW2, W_s + OFFB_IW1, j > 0, iW3, iB3, iW2, iB2, iW1, iB1, in_i, map_w1);
+      const bool more = j + 1 < M;
+      ok = layer_backward(
+          dz3, w3_i, W_s + OFFB_IW2, W_s + OFFB_IW1, j > 0, iW3, iB3, iW2, iB2, iW1, iB1, in_i, map_w1,
+          [&] {
+            if (!more) return;
+            wj = cosine_direction_fast(n2, m.seed, dir_counter(q, M, 2 + j));
+            store_pe_tmem(X_w, wj);
+          },
+          [&](uint32_t one) {
+            if (more) mma_layer1(one, D_t, X_t, W_s + OFFB_IW1);
+          });
     }
     if (!ok) break;
     lo2 = lo2 * sM;
@@ -565,7 +582,7 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
       dy[5] = da2.z * a2.z * (1.0f - a2.z);
       dy[6] = dr2 * 0.91f * s6 * (1.0f - s6);
       if (!layer_backward(dy, w3_b, W_s + OFFB_BW2, W_s + OFFB_BW1, M > 0, gB.w3(), gB.b3(), gB.w2(), gB.b2(), gB.w1(),
-                          gB.b1(), lf, map_w1b))
+                          gB.b1(), lf, map_w1b, nothing, no_ride))
         break;
     }
 
@@ -620,7 +637,8 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
     store_primary_hi(fpix, ps, X_w, wi);   // the layer-1 input's hi parts back into X
     {
       // as layer_backward, with the primary point's df accumulated into F afresh
-      if (!layer_backward(dzp, w3_i, W_s + OFFB_IW2, W_s + OFFB_IW1, false, iW3, iB3, iW2, iB2, iW1, iB1, in_i, map_w1))
+      if (!layer_backward(dzp, w3_i, W_s + OFFB_IW2, W_s + OFFB_IW1, false, iW3, iB3, iW2, iB2, iW1, iB1, in_i, map_w1,
+                          nothing, no_ride))
         break;
     }
 
