@@ -267,8 +267,8 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
   int abort = 0;
 
   // One MMA round trip (as in the forward): the rows' TMEM stores and staging-tile stores are made
-  // visible to the tensor core, the warpgroup votes on `abort`, thread 0 issues and commits, and every
-  // thread waits on the mbarrier with a bound.
+  // visible to the tensor core, the warpgroup votes on `abort`, an elected lane of warp 0 issues and
+  // commits, and every thread waits on the mbarrier with a bound.
   auto run_mma = [&](auto issue) -> bool {
     tmem_st_wait();
     fence_async_smem();

@@ -359,7 +359,7 @@ cudaError_t prepare_backward_fp32() {
 
 cudaError_t launch_backward_fp32(const ModelDesc& m, const rt_gbuffer& gb, int P, long long offset, const float4* dL,
                                  float* g_table, float* g_brdf, float* g_irt, int num_sms, cudaStream_t s) {
-  const int need = (P + kAdjWarps - 1) / kAdjWarps;
+  const int need = (int)(((long long)P + kAdjWarps - 1) / kAdjWarps);
   const int grid = need < num_sms ? need : num_sms;
   backward_fp32_kernel<<<grid, kAdjThreads, kBSmem, s>>>(m, gb, P, offset, dL, g_table, g_brdf, g_irt);
   return cudaGetLastError();

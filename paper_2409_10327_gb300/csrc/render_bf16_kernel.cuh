@@ -145,8 +145,8 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
   int abort = 0;
   if (t < kCarrySlots * NL) carry_s[t] = make_float4(0.f, 0.f, 0.f, 0.f);
 
-  // One MMA round trip: barrier with an abort vote, issue by thread 0,
-  // commit, bounded wait.  A wait that gives up only raises `abort`; the
+  // One MMA round trip: barrier with an abort vote, issue and commit by an
+  // elected lane of warp 0, bounded wait.  A wait that gives up only raises `abort`; the
   // vote at the next round trip then stops all 128 threads together, so the
   // warpgroup never splits across barriers.
   uint32_t pending_phase = 0;

@@ -17,8 +17,9 @@ constexpr int kIrtOut = 2;      // [visibility logit, depth logit]
 
 // Packed FP32 weight image (floats).  Weights are stored transposed,
 // [in][out] with out = 64 contiguous, so that one k step of a warp GEMM
-// reads a 64-wide row.  Rows beyond the true fan-in are zero.  The image is
-// copied verbatim into shared memory by the fused kernels.
+// reads a 64-wide row.  Rows beyond the true fan-in are zero.  The FP32
+// kernels copy the parts they need into shared memory verbatim, or split into
+// bf16 parts (tc_split.cuh).
 constexpr int OFF_IW1F = 0;                      // I, layer 1, feature rows   [32][64]
 constexpr int OFF_IW1P = OFF_IW1F + 32 * 64;     // I, layer 1, PE rows        [32][64]
 constexpr int OFF_IB1 = OFF_IW1P + 32 * 64;      // [64]

@@ -25,9 +25,10 @@ def lib():
     return binding
 
 
-# N < 4: more pixels in a tile than feature slots; 4: as many as there can be; 33, 130: pixels that start and end
-# anywhere in a tile and span several
-@pytest.mark.parametrize("n_dirs, P", [(1, 300), (2, 131), (3, 700), (4, 129), (33, 11), (130, 5)])
+# 1 .. 14: more pixels in a tile than shared feature slots; 15: as many, or one more, by where the tile starts; 16, 33,
+# 130: fewer, with pixels that start and end anywhere in a tile or span several
+@pytest.mark.parametrize("n_dirs, P", [(1, 300), (2, 131), (3, 700), (4, 129), (14, 40), (15, 61), (16, 33), (33, 11),
+                                       (130, 5)])
 def test_frame_tiles(lib, n_dirs, P):
     cfg = helpers.small_cfg(n_dirs=n_dirs, m_dirs=3)
     sc, gb = helpers.scene_arrays(cfg, 4, bias=0.2, n_pixels=P)
@@ -81,3 +82,35 @@ def test_denoise_blocks(lib, h, w, iters, sigma_n):
     got = test_gpu_denoise._run(lib, c, z, n, iterations=iters, sigma_n=sigma_n)
     ref_c, ref_v = oden.svgf(c, z, n, iterations=iters, sigma_n=sigma_n)
     test_gpu_denoise._check(got, ref_c, ref_v)
+
+
+# 16-byte accesses where every buffer allows them, 4-byte ones otherwise; sizes off four
+@pytest.mark.parametrize("n", [1, 3, 4, 1003, 300001])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_adam_alignment(lib, n, shift):
+    g = torch.Generator(device="cuda").manual_seed(n)
+    base = [torch.rand(n + 1, generator=g, device="cuda") for _ in range(4)]
+    one = [b[:n].clone() for b in base]                       # aligned
+    two = [torch.cat([b.new_zeros(shift), b[:n]])[shift:] for b in base]
+    lib.adam_step(*one, step=3, lr=0.01, weight_decay=1e-2)
+    lib.adam_step(*two, step=3, lr=0.01, weight_decay=1e-2)
+    for a, b in zip(one, two):
+        assert torch.equal(a, b)
+    # the update from its definition, in 64 bits; each of the few operations rounds once
+    p, d, m, v = (b[:n].double() for b in base)
+    d = d + 1e-2 * p
+    m, v = 0.9 * m + 0.1 * d, 0.999 * v + 0.001 * d * d
+    p = p - 0.01 * (m / (1 - 0.9 ** 3)) / ((v / (1 - 0.999 ** 3)).sqrt() + 1e-8)
+    torch.testing.assert_close(one[0].double(), p, rtol=1e-5, atol=1e-6)
+
+
+# features go out as pairs where the buffer allows 8-byte stores
+def test_encode_alignment(lib):
+    cfg = helpers.small_cfg(levels=5)
+    r = helpers.renderer_for(cfg, scenegen.make_scene(cfg, 0))
+    pos = torch.rand(77, 4, device="cuda") * 2.4 - 1.2
+    want = r.encode(pos)
+    buf = torch.full((77 * 10 + 1,), float("nan"), device="cuda")
+    assert lib.LIB.rt_encode(r.ctx, lib._ptr(pos), 77, lib._ptr(buf[1:]), None, None, None) == lib.RT_OK
+    torch.cuda.synchronize()
+    assert torch.equal(buf[1:].view(77, 10), want)
