@@ -33,6 +33,7 @@ struct rt_ctx {
 namespace {
 
 constexpr int64_t kMaxP = 2147483647LL;
+constexpr int kDoneWord = 32;   // words 32 and 33 of the status block: rt_set_params' count of finished rows
 
 bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
@@ -292,13 +293,11 @@ rt_status rt_set_params(rt_ctx* ctx, const void* table, const float* brdf_w, con
   ctx->env = env;
   const int lf = ctx->cfg.levels * ctx->cfg.feat_dim;
   cudaStream_t s = (cudaStream_t)stream;
-  rt_status st = cuda_status(launch_repack(brdf_w, irt_w, lf, ctx->wpack, s));
-  if (st == RT_OK)
-    st = cuda_status(launch_env_cdf(reinterpret_cast<const float4*>(env), ctx->cfg.env_h, ctx->cfg.env_w, ctx->cdf,
-                                    ctx->cdf + (ctx->cfg.env_h + 1), guide_m_of(ctx->cdf, ctx->cfg),
-                                    guide_shift(ctx->cfg.env_h), guide_c_of(ctx->cdf, ctx->cfg),
-                                    guide_shift(ctx->cfg.env_w), s));
-  if (st == RT_OK) st = cuda_status(launch_repack_bf16(ctx->wpack, ctx->wbf16, s));
+  const rt_status st = cuda_status(launch_set_params(
+      brdf_w, irt_w, lf, ctx->wpack, ctx->wbf16, reinterpret_cast<const float4*>(env), ctx->cfg.env_h, ctx->cfg.env_w,
+      ctx->cdf, ctx->cdf + (ctx->cfg.env_h + 1), guide_m_of(ctx->cdf, ctx->cfg), guide_shift(ctx->cfg.env_h),
+      guide_c_of(ctx->cdf, ctx->cfg), guide_shift(ctx->cfg.env_w),
+      reinterpret_cast<unsigned long long*>(ctx->status + kDoneWord), s));
   if (st != RT_OK) return st;
   // Host copy of the output layers for the BF16 kernel's parameters: the two spans of the packed image that hold
   // them (I's W3 and b3; B's W3 and b3) as two rows of one strided copy, 4 KB instead of the image's 61.

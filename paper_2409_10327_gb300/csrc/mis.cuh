@@ -6,7 +6,7 @@
 // sampling, (n . w)+ / (n_L p_L(w) + n_G p_G(w)) * N / pi, rides on its BRDF
 // (mis_weighted_brdf).
 //   light: texel (r, c) by inverting the float32 CDFs of the bound
-//     environment map (built by env_cdf kernels in the same order as their
+//     environment map (built by rt_set_params in the same order as their
 //     float32 reference), then a point uniform in (phi, theta) inside the
 //     texel: p_L = p_texel / (dphi dtheta sin(theta));
 //   GGX: Heitz's visible-normal sampler (alpha = r^2) in Duff et al.'s frame

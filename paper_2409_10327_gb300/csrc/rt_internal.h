@@ -132,7 +132,6 @@ cudaError_t launch_sample(const ModelDesc& m, const float4* normal, int P, int l
                           float4* dirs, cudaStream_t s);
 cudaError_t launch_shade(const ModelDesc& m, const rt_gbuffer& pts, int P, int level, long long offset,
                          const float* vis, const float4* lin, float4* out, cudaStream_t s);
-cudaError_t launch_repack_bf16(const float* wpack, uint8_t* wbf16, cudaStream_t s);
 // the direction-chunk tile shapes (m.dpt 32 / 64), soft visibility, one launch of nl lights
 cudaError_t prepare_render_bf16_chunked();
 cudaError_t launch_render_bf16_chunked(int nl, int wg, const ModelDesc& m, const HeadParams& hp, const rt_gbuffer& gb,
@@ -160,8 +159,10 @@ cudaError_t launch_distill_fp32(const ModelDesc& m, const float4* pos, const flo
                                 float* loss, float* g_table, float* g_brdf, float* g_irt, int num_sms, cudaStream_t s);
 cudaError_t launch_adam(float* p, const float* g, float* m1, float* m2, long long n, float lr, float b1, float b2,
                         float eps, float wd, float bc1, float bc2, int num_sms, cudaStream_t s);
-cudaError_t launch_env_cdf(const float4* env, int H, int W, float* cdf_m, float* cdf_c, int* guide_m, int gm_shift,
-                           int* guide_c, int gc_shift, cudaStream_t s);
+// both weight images and the texel CDFs of the map; done: a device counter of finished rows, zero at first
+cudaError_t launch_set_params(const float* brdf_w, const float* irt_w, int lf, float* wpack, uint8_t* wbf16,
+                              const float4* env, int H, int W, float* cdf_m, float* cdf_c, int* guide_m, int gm_shift,
+                              int* guide_c, int gc_shift, unsigned long long* done, cudaStream_t s);
 // smallest s with 2^s >= n (n >= 1): the cutpoint tables have 2^s entries
 inline int guide_shift(int n) {
   int s = 0;

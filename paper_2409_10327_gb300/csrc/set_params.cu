@@ -1,5 +1,11 @@
-// Texel distribution of the bound environment map for the light strategy of
-// the MIS primary sampler (Sec. 4.1): luminance 0.2126 R + 0.7152 G +
+// rt_set_params' device work in one launch: the FP32 and BF16 weight images,
+// and the texel distribution of the bound environment map.  They are
+// independent (the BF16 image is formed from the blobs, not from the FP32
+// image), so the rows of the map and both images share a grid, and the CTA
+// that finishes the last row builds the marginal; as four dependent launches
+// they took 19 us for a 256 x 512 map, most of it launch latency and drain.
+//
+// Texel distribution for the light strategy of the MIS primary sampler (Sec. 4.1): luminance 0.2126 R + 0.7152 G +
 // 0.0722 B, negative parts clipped, plus 1e-6; conditional CDFs along each
 // row and a marginal CDF over rows.  The inversion of these CDFs decides
 // integers, so they are built in float32 with every product and sum
@@ -17,11 +23,14 @@
 // With the chain in global memory (one thread per row, a dependent load and a
 // strided store per texel) a 256 x 512 map took 403 us and its marginal 34 us.
 #include "mis.cuh"
+#include "repack.cuh"
 
 namespace rtk {
 namespace {
 
 constexpr int kCdfThreads = 128;
+constexpr int kPackBlocks = (WPACK_FLOATS + kCdfThreads - 1) / kCdfThreads;
+constexpr int kBf16Blocks = (WBF16_BYTES / 2 + kCdfThreads - 1) / kCdfThreads;
 
 // v[0..n) -> its running sums, in index order, each rounded to float32; the last one is the total.
 __device__ __forceinline__ void running_sum(float* v, int n) {
@@ -76,33 +85,48 @@ __device__ __forceinline__ void finish_cdf(float* v, int n, float* __restrict__ 
   }
 }
 
-// CTA r: the conditional CDF of row r, its cutpoints, and the row's total into cdf_m[r + 1].
+// CTA r < H: the conditional CDF of row r, its cutpoints, and the row's total into cdf_m[r + 1]; the CTA that finishes
+// last (every H-th count of *done, which only grows) turns the totals into the marginal CDF and answers its cutpoints.
+// Further CTAs: kCdfThreads elements of the FP32 image each, then of the BF16 image.
 __global__ void __launch_bounds__(kCdfThreads)
-env_cdf_rows_kernel(const float4* __restrict__ env, int W, float* __restrict__ cdf_m, float* __restrict__ cdf_c,
-                    int* __restrict__ guide_c, int gc_shift) {
+set_params_kernel(const float* __restrict__ bw, const float* __restrict__ iw, int lf, float* __restrict__ wpack,
+                  uint8_t* __restrict__ wbf16, const float4* __restrict__ env, int H, int W, float* cdf_m,
+                  float* __restrict__ cdf_c, int* __restrict__ guide_m, int gm_shift, int* __restrict__ guide_c,
+                  int gc_shift, unsigned long long* done) {
   extern __shared__ float4 cdf_smem4[];
   float* v = reinterpret_cast<float*>(cdf_smem4);
   const int r = blockIdx.x;
+  if (r >= H) {
+    int e = (r - H) * kCdfThreads + threadIdx.x;
+    if (e < kPackBlocks * kCdfThreads) {
+      if (e < WPACK_FLOATS) wpack[e] = packed_value(bw, iw, lf, e);
+      return;
+    }
+    e -= kPackBlocks * kCdfThreads;
+    if (e < WBF16_BYTES / 2)
+      reinterpret_cast<__nv_bfloat16*>(wbf16)[e] =
+          bf16_image_value(2 * e, [&](int k) { return packed_value(bw, iw, lf, k); });
+    return;
+  }
   for (int c = threadIdx.x; c < W; c += kCdfThreads) {
     const float4 e = env[(size_t)r * W + c];
     const float lum = __fadd_rn(__fadd_rn(__fmul_rn(e.x, 0.2126f), __fmul_rn(e.y, 0.7152f)), __fmul_rn(e.z, 0.0722f));
     v[c] = __fadd_rn(fmaxf(lum, 0.0f), 1e-6f);
   }
   __syncthreads();
+  __shared__ uint32_t last;
   if (threadIdx.x == 0) {
     running_sum(v, W);
-    cdf_m[r + 1] = v[W - 1];   // turned into the marginal CDF below
+    __stcg(cdf_m + r + 1, v[W - 1]);   // turned into the marginal CDF by the last CTA
+    __threadfence();
+    last = (atomicAdd(done, 1ull) + 1ull) % (unsigned)H == 0;
   }
   __syncthreads();
   finish_cdf(v, W, cdf_c + (size_t)r * (W + 1), guide_c + ((size_t)r << gc_shift), gc_shift);
-}
-
-// One CTA: the marginal CDF of the row totals in cdf_m[1..H], in place, and its cutpoints.
-__global__ void __launch_bounds__(kCdfThreads)
-env_cdf_marginal_kernel(int H, float* __restrict__ cdf_m, int* __restrict__ guide_m, int gm_shift) {
-  extern __shared__ float4 cdf_smem4[];
-  float* v = reinterpret_cast<float*>(cdf_smem4);
-  for (int r = threadIdx.x; r < H; r += kCdfThreads) v[r] = cdf_m[r + 1];
+  if (!last) return;
+  __threadfence();   // the other rows' totals are visible
+  __syncthreads();   // v is read
+  for (int k = threadIdx.x; k < H; k += kCdfThreads) v[k] = __ldcg(cdf_m + k + 1);
   __syncthreads();
   if (threadIdx.x == 0) running_sum(v, H);
   __syncthreads();
@@ -111,13 +135,13 @@ env_cdf_marginal_kernel(int H, float* __restrict__ cdf_m, int* __restrict__ guid
 
 }  // namespace
 
-cudaError_t launch_env_cdf(const float4* env, int H, int W, float* cdf_m, float* cdf_c, int* guide_m, int gm_shift,
-                           int* guide_c, int gc_shift, cudaStream_t s) {
-  // a row of at most 8192 floats fits the 48 KB of shared memory that need no opt-in
-  env_cdf_rows_kernel<<<H, kCdfThreads, ((size_t)W + 3) / 4 * 16, s>>>(env, W, cdf_m, cdf_c, guide_c, gc_shift);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  env_cdf_marginal_kernel<<<1, kCdfThreads, ((size_t)H + 3) / 4 * 16, s>>>(H, cdf_m, guide_m, gm_shift);
+cudaError_t launch_set_params(const float* brdf_w, const float* irt_w, int lf, float* wpack, uint8_t* wbf16,
+                              const float4* env, int H, int W, float* cdf_m, float* cdf_c, int* guide_m, int gm_shift,
+                              int* guide_c, int gc_shift, unsigned long long* done, cudaStream_t s) {
+  // a row or column of at most 8192 floats fits the 48 KB of shared memory that need no opt-in
+  const size_t smem = ((size_t)(H > W ? H : W) + 3) / 4 * 16;
+  set_params_kernel<<<H + kPackBlocks + kBf16Blocks, kCdfThreads, smem, s>>>(
+      brdf_w, irt_w, lf, wpack, wbf16, env, H, W, cdf_m, cdf_c, guide_m, gm_shift, guide_c, gc_shift, done);
   return cudaGetLastError();
 }
 

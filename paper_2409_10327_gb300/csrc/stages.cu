@@ -4,59 +4,15 @@
 // what the fused kernel computes per sample and give each stage its own parity
 // check.
 #include "device_common.cuh"
+#include "repack.cuh"
 
 namespace rtk {
 
-// ---- weight repacking ------------------------------------------------------
-// Canonical blob (per MLP): W1 [64][in], b1 [64], W2 [64][64], b2 [64],
-// W3 [out][64], b3 [out].  Output: the transposed image of rt_internal.h.
+// ---- weight repacking on its own (rt_render_frame_static; rt_set_params does it with the rest) ----
 __global__ void repack_kernel(const float* __restrict__ bw, const float* __restrict__ iw, int lf,
                               float* __restrict__ out) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= WPACK_FLOATS) return;
-  const int in_i = lf + kPE;
-  // I blob offsets
-  const int iW1 = 0, iB1 = iW1 + 64 * in_i, iW2 = iB1 + 64, iB2 = iW2 + 64 * 64, iW3 = iB2 + 64, iB3 = iW3 + 2 * 64;
-  // B blob offsets
-  const int bW1 = 0, bB1 = bW1 + 64 * lf, bW2 = bB1 + 64, bB2 = bW2 + 64 * 64, bW3 = bB2 + 64, bB3 = bW3 + 7 * 64;
-  float v = 0.0f;
-  if (e < OFF_IW1P) {                         // I W1, feature rows [k][c]
-    const int k = (e - OFF_IW1F) / 64, c = (e - OFF_IW1F) % 64;
-    if (k < lf) v = iw[iW1 + c * in_i + k];
-  } else if (e < OFF_IB1) {                   // I W1, PE rows
-    const int k = (e - OFF_IW1P) / 64, c = (e - OFF_IW1P) % 64;
-    if (k < kPE) v = iw[iW1 + c * in_i + lf + k];
-  } else if (e < OFF_IW2) {
-    v = iw[iB1 + (e - OFF_IB1)];
-  } else if (e < OFF_IB2) {
-    const int k = (e - OFF_IW2) / 64, c = (e - OFF_IW2) % 64;
-    v = iw[iW2 + c * 64 + k];
-  } else if (e < OFF_IW3) {
-    v = iw[iB2 + (e - OFF_IB2)];
-  } else if (e < OFF_IB3) {
-    const int k = (e - OFF_IW3) / 2, c = (e - OFF_IW3) % 2;
-    v = iw[iW3 + c * 64 + k];
-  } else if (e < OFF_BW1) {
-    const int c = e - OFF_IB3;
-    if (c < 2) v = iw[iB3 + c];
-  } else if (e < OFF_BB1) {
-    const int k = (e - OFF_BW1) / 64, c = (e - OFF_BW1) % 64;
-    if (k < lf) v = bw[bW1 + c * lf + k];
-  } else if (e < OFF_BW2) {
-    v = bw[bB1 + (e - OFF_BB1)];
-  } else if (e < OFF_BB2) {
-    const int k = (e - OFF_BW2) / 64, c = (e - OFF_BW2) % 64;
-    v = bw[bW2 + c * 64 + k];
-  } else if (e < OFF_BW3) {
-    v = bw[bB2 + (e - OFF_BB2)];
-  } else if (e < OFF_BB3) {
-    const int k = (e - OFF_BW3) / 8, c = (e - OFF_BW3) % 8;
-    if (c < 7) v = bw[bW3 + c * 64 + k];
-  } else {
-    const int c = e - OFF_BB3;
-    if (c < 7) v = bw[bB3 + c];
-  }
-  out[e] = v;
+  if (e < WPACK_FLOATS) out[e] = packed_value(bw, iw, lf, e);
 }
 
 cudaError_t launch_repack(const float* brdf_w, const float* irt_w, int lf, float* wpack, cudaStream_t s) {
