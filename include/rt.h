@@ -376,6 +376,14 @@ rt_status rt_probe_ffma(int32_t iters, int32_t blocks, float* sink, void* stream
  * K must be a perfect square (1..65536); P * K < 2^31. */
 rt_status rt_distill_dirs(rt_ctx* ctx, int64_t P, int32_t K, int64_t ray_offset, float* dirs, void* stream);
 
+/* The teacher's visibility and depth for rt_distill_backward: rt_trace's values,
+ * by FP32 FMA chains in a fixed order, at the front-facing directions only
+ * (dirs . normal > 0; the others take no part in the loss: visibility 0, depth
+ * near_t).  feat [P][L*F] (rt_encode), dirs [P][K][4], normal [P][4],
+ * vis and depth [P][K], all device; K <= 65536, P K < 2^31. */
+rt_status rt_distill_targets(rt_ctx* ctx, const float* feat, const float* dirs, const float* normal, int64_t P, int32_t K,
+                             float* vis, float* depth, void* stream);
+
 /* ACCUMULATES the gradient of the per-head distillation loss of the student
  * ctx (RT_FP32 only, else RT_ERR_UNSUPPORTED) into g_table [L][T][F],
  * g_brdf and g_irt (float, blob layouts; the caller zeroes them), and adds

@@ -30,6 +30,7 @@ EXPORTS = ["rt_status_str", "rt_config_default", "rt_config_validate", "rt_level
            "rt_set_params", "rt_check", "rt_encode", "rt_decode", "rt_trace", "rt_sample", "rt_shade",
            "rt_render_frame", "rt_backward", "rt_render_frame_static", "rt_render_frame_multi", "rt_tune",
            "rt_tuned_shape", "rt_set_launch_shape", "rt_tuned_tile_shape", "rt_set_tile_shape", "rt_denoise", "rt_distill_dirs",
+           "rt_distill_targets",
            "rt_distill_backward", "rt_adam_step", "rt_selftest_wait", "rt_debug_fail_alloc",
            "rt_probe_gather", "rt_probe_ffma"]
 
@@ -90,6 +91,7 @@ def _load() -> ctypes.CDLL:
         "rt_set_tile_shape": (I32, [P, I32]),
         "rt_denoise": (I32, [I32, I32, P, P, P, I32, F32, F32, F32, P, P, P]),
         "rt_distill_dirs": (I32, [P, I64, I32, I64, P, P]),
+        "rt_distill_targets": (I32, [P, P, P, P, I64, I32, P, P, P]),
         "rt_distill_backward": (I32, [P, P, P, I64, I32, P, P, P, P, P, P, P, P, P]),
         "rt_adam_step": (I32, [P, P, P, P, I64, F32, F32, F32, F32, F32, I32, P]),
         "rt_selftest_wait": (I32, [P, I64, P]),
@@ -340,6 +342,15 @@ class Renderer:
         dirs = torch.empty(P, K, 4, device="cuda", dtype=torch.float32)
         _check("rt_distill_dirs", LIB.rt_distill_dirs(self.ctx, P, K, ray_offset, _ptr(dirs), _stream()))
         return dirs
+
+    def distill_targets(self, feat: torch.Tensor, dirs: torch.Tensor, normal: torch.Tensor):
+        """Visibility and depth [P, K] at the front-facing directions (elsewhere 0 and the near depth)."""
+        P, K = dirs.shape[0], dirs.shape[1]
+        vis = torch.empty(P, K, device=dirs.device, dtype=torch.float32)
+        depth = torch.empty_like(vis)
+        _check("rt_distill_targets", LIB.rt_distill_targets(self.ctx, _ptr(feat), _ptr(dirs), _ptr(normal), P, K, _ptr(vis),
+                                                            _ptr(depth), _stream()))
+        return vis, depth
 
     def distill_backward(self, pos: torch.Tensor, normal: torch.Tensor, dirs: torch.Tensor, brdf_t: torch.Tensor,
                          vis_t: torch.Tensor, depth_t: torch.Tensor, loss: Optional[torch.Tensor],

@@ -603,6 +603,20 @@ rt_status rt_distill_dirs(rt_ctx* ctx, int64_t P, int32_t K, int64_t ray_offset,
                                          (cudaStream_t)stream));
 }
 
+rt_status rt_distill_targets(rt_ctx* ctx, const float* feat, const float* dirs, const float* normal, int64_t P, int32_t K,
+                             float* vis, float* depth, void* stream) {
+  rt_status st = check_ctx(ctx);
+  if (st != RT_OK) return st;
+  if (P < 0 || K < 1 || K > 65536 || P * (int64_t)K > kMaxP) return RT_ERR_INVALID_ARG;
+  if (P == 0) return RT_OK;
+  if (feat == nullptr || !aligned(feat, 4) || !check_plane(dirs) || !check_plane(normal) || vis == nullptr ||
+      !aligned(vis, 4) || depth == nullptr || !aligned(depth, 4))
+    return RT_ERR_INVALID_ARG;
+  return cuda_status(launch_distill_targets(model_desc(ctx), feat, reinterpret_cast<const float4*>(dirs),
+                                            reinterpret_cast<const float4*>(normal), (int)P, K, vis, depth, ctx->num_sms,
+                                            (cudaStream_t)stream));
+}
+
 rt_status rt_distill_backward(rt_ctx* ctx, const float* pos, const float* normal, int64_t P, int32_t K,
                               const float* dirs, const float* brdf_t, const float* vis_t, const float* depth_t,
                               float* loss, float* g_table, float* g_brdf, float* g_irt, void* stream) {

@@ -11,7 +11,7 @@
 //   (w . n > 0) and then over points.
 //
 // Work, in two phases of one persistent launch.  I phase: a unit is one
-// point and up to 256 of its directions; the warp encodes f = H(x), counts
+// point and up to 256 of its directions (blocks of 32 in turn); the warp encodes f = H(x), counts
 // the point's front-facing directions, lists the unit's (the others carry no
 // loss) and walks the list 32 at a time (lane = direction): I forward, the
 // head gradients, I's adjoint with the layer-1 f part shared by the unit's
@@ -45,6 +45,16 @@ static_assert(DB_H1 % 4 == 0 && DB_H2 % 4 == 0 && DB_H2 == DB_H1 + kActStride &&
                   DB_FLOATS % 4 == 0,
               "float4 alignment");
 
+// Direction j of a point's unit `unit` of nch: the units take blocks of 32 directions in turn.  Stratified directions
+// run over the sphere in bands, so a unit of consecutive ones would be all front-facing or all back-facing, and with
+// nch dividing the number of warps a warp would meet the same band at every point (2,048 x 1,024: 1.47 ms so, 0.98 ms
+// in turn).
+__device__ __forceinline__ int unit_dir(int unit, int nch, int j) { return ((unit + nch * (j >> 5)) << 5) + (j & 31); }
+
+// w . n > 0 with every operation pinned: the teacher's and the student's kernels have to agree on it.
+__device__ __forceinline__ bool front_facing(float4 w, f3 n) {
+  return __fmaf_rn(w.z, n.z, __fmaf_rn(w.y, n.y, __fmul_rn(w.x, n.x))) > 0.0f;
+}
 __device__ __forceinline__ float sgnf(float d) { return d > 0.0f ? 1.0f : (d < 0.0f ? -1.0f : 0.0f); }
 
 __global__ void distill_dirs_kernel(long long PK, int K, int S, long long ray_offset, uint64_t seed,
@@ -63,6 +73,89 @@ __global__ void distill_dirs_kernel(long long PK, int K, int S, long long ray_of
   float sp, cp;
   sincospif(2.0f * u2, &sp, &cp);
   dirs[e] = make_float4(rho * cp, rho * sp, z, 0.0f);
+}
+
+// ---- the teacher's visibility and depth at the front-facing directions ------
+// I as the student's kernel evaluates it: FP32 FMA chains in a fixed order, for
+// the loss takes signs (hit or not, deeper or not) that a last bit can turn.
+// The other directions, half of them on average, have no part in the loss and
+// get vis 0 and the near depth: 2,048 x 1,024 take 0.32 ms, rt_trace's
+// tensor-core rows over all of them 0.19 ms.  Units and lists as in the I phase;
+// one in-place activation buffer per warp, so twelve warps.
+constexpr int kTgWarps = 12;
+constexpr int kTgThreads = 32 * kTgWarps;
+constexpr int TG_ACT = 0, TG_FP = kActStride, TG_AP = TG_FP + 32, TG_LIST = TG_AP + 64;
+constexpr int TG_FLOATS = TG_LIST + kUnitDirs / 2;
+constexpr size_t kTgSmem = (size_t)(OFF_BW1 + kTgWarps * TG_FLOATS) * sizeof(float);
+static_assert(OFF_BW1 % 4 == 0 && TG_FLOATS % 4 == 0 && kTgSmem <= 232448, "float4 alignment, one CTA per SM");
+
+__global__ void __launch_bounds__(kTgThreads, 1)
+distill_targets_kernel(ModelDesc m, const float* __restrict__ feat, const float4* __restrict__ dirs,
+                       const float4* __restrict__ nrm4, int P, int K, float* __restrict__ vis,
+                       float* __restrict__ depth) {
+  extern __shared__ float4 smem4[];
+  float* sw = reinterpret_cast<float*>(smem4);
+  for (int i = threadIdx.x; i < OFF_BW1 / 4; i += kTgThreads) smem4[i] = __ldg(reinterpret_cast<const float4*>(m.wpack) + i);
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rg = lane >> 3, cg = lane & 7;
+  float* act = sw + OFF_BW1 + warp * TG_FLOATS + TG_ACT;
+  float* fP = act + TG_FP;
+  float* aP = act + TG_AP;
+  uint16_t* list = reinterpret_cast<uint16_t*>(act + TG_LIST);
+  const int nch = (K + kUnitDirs - 1) / kUnitDirs;
+  const long long units = (long long)P * nch;
+  for (long long u = (long long)blockIdx.x * kTgWarps + warp; u < units; u += (long long)gridDim.x * kTgWarps) {
+    const int p = (int)(u / nch);
+    const int unit = (int)(u - (long long)p * nch);
+    const f3 n = xyz(nrm4[p]);
+    fP[lane] = lane < m.lf ? feat[(size_t)p * m.lf + lane] : 0.0f;
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = lane + 32 * h;
+      float acc = sw[OFF_IB1 + c];
+      for (int k = 0; k < m.lfp; ++k) acc = fmaf(fP[k], sw[OFF_IW1F + k * 64 + c], acc);
+      aP[c] = acc;
+    }
+    int nlist = 0;
+#pragma unroll 4
+    for (int j0 = 0; unit_dir(unit, nch, j0) < K; j0 += 32) {
+      const int k = unit_dir(unit, nch, j0 + lane);
+      const bool ff = k < K && front_facing(dirs[(size_t)p * K + k], n);
+      if (k < K && !ff) {
+        vis[(size_t)p * K + k] = 0.0f;
+        depth[(size_t)p * K + k] = m.near_t;
+      }
+      const unsigned bal = __ballot_sync(0xffffffffu, ff);
+      if (ff) list[nlist + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(j0 + lane);
+      nlist += __popc(bal);
+    }
+    __syncwarp();
+    for (int r0 = 0; r0 < nlist; r0 += 32) {
+      const bool ff = r0 + lane < nlist;
+      const size_t e = (size_t)p * K + unit_dir(unit, nch, (int)list[ff ? r0 + lane : r0]);
+      Tile acc;
+      store_pe(act, xyz(dirs[e]), lane);
+      __syncwarp();
+      zero(acc);
+      warp_gemm<kPEPad - 4>(act, sw + OFF_IW1P, acc, rg, cg);
+      __syncwarp();
+      store_relu_colbias(act, acc, aP, rg, cg);
+      __syncwarp();
+      zero(acc);
+      warp_gemm<kHidden>(act, sw + OFF_IW2, acc, rg, cg);
+      __syncwarp();
+      store_relu_colbias(act, acc, sw + OFF_IB2, rg, cg);
+      __syncwarp();
+      const float2 z = irt_head(act, sw, lane);
+      if (ff) {
+        vis[e] = sigmoidf_(z.x);
+        depth[e] = depth_from_logit(z.y, m.near_t, m.far_t);
+      }
+      __syncwarp();
+    }
+  }
 }
 
 __global__ void __launch_bounds__(kAdjThreads, 1)
@@ -103,8 +196,7 @@ distill_fp32_kernel(ModelDesc m, const float4* __restrict__ pos4, const float4* 
   for (long long u = (long long)blockIdx.x * kAdjWarps + warp; u < units; u += (long long)gridDim.x * kAdjWarps) {
     {
       const int p = (int)(u / nch);
-      const int kb = (int)(u - (long long)p * nch) * kUnitDirs;
-      const int ke = min(K, kb + kUnitDirs);
+      const int unit = (int)(u - (long long)p * nch);
       const f3 x = xyz(pos4[p]);
       const f3 n = xyz(nrm4[p]);
       {
@@ -133,11 +225,11 @@ distill_fp32_kernel(ModelDesc m, const float4* __restrict__ pos4, const float4* 
 #pragma unroll 4   // the loads of four steps in flight
       for (int k0 = 0; k0 < K; k0 += 32) {
         const int k = k0 + lane;
-        const bool ff = k < K && dot(xyz(dirs[(size_t)p * K + k]), n) > 0.0f;
+        const bool ff = k < K && front_facing(dirs[(size_t)p * K + k], n);
         const unsigned bal = __ballot_sync(0xffffffffu, ff);
         cnt += __popc(bal);
-        if (k0 >= kb && k0 < ke) {
-          if (ff) list[nlist + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(k - kb);
+        if ((k0 >> 5) % nch == unit) {
+          if (ff) list[nlist + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(((k0 >> 5) / nch << 5) + lane);
           nlist += __popc(bal);
         }
       }
@@ -146,7 +238,7 @@ distill_fp32_kernel(ModelDesc m, const float4* __restrict__ pos4, const float4* 
       __syncwarp();
       for (int r0 = 0; r0 < nlist; r0 += 32) {
         const bool ff = r0 + lane < nlist;
-        const int k = kb + (int)list[ff ? r0 + lane : r0];
+        const int k = unit_dir(unit, nch, (int)list[ff ? r0 + lane : r0]);
         const f3 w = xyz(dirs[(size_t)p * K + k]);
         Tile acc;
         store_pe(PEb, w, lane);
@@ -339,6 +431,9 @@ __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, 
 }  // namespace
 
 cudaError_t prepare_distill() {
+  const cudaError_t e =
+      cudaFuncSetAttribute(distill_targets_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTgSmem);
+  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(distill_fp32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDSmem);
 }
 
@@ -347,6 +442,15 @@ cudaError_t launch_distill_dirs(int P, int K, long long ray_offset, uint64_t see
   while ((S + 1) * (S + 1) <= K) ++S;
   const long long PK = (long long)P * K;
   distill_dirs_kernel<<<(unsigned)((PK + 255) / 256), 256, 0, s>>>(PK, K, S, ray_offset, seed, dirs);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_distill_targets(const ModelDesc& m, const float* feat, const float4* dirs, const float4* nrm, int P,
+                                   int K, float* vis, float* depth, int num_sms, cudaStream_t s) {
+  const long long units = (long long)P * ((K + kUnitDirs - 1) / kUnitDirs);
+  const long long need = (units + kTgWarps - 1) / kTgWarps;
+  const int grid = (int)(need < num_sms ? need : num_sms);
+  distill_targets_kernel<<<grid, kTgThreads, kTgSmem, s>>>(m, feat, dirs, nrm, P, K, vis, depth);
   return cudaGetLastError();
 }
 

@@ -154,6 +154,8 @@ cudaError_t launch_render_fp32(const ModelDesc& m, const rt_gbuffer& gb, int P, 
                                float4* out, int num_sms, cudaStream_t s);
 cudaError_t prepare_distill();
 cudaError_t launch_distill_dirs(int P, int K, long long ray_offset, uint64_t seed, float4* dirs, cudaStream_t s);
+cudaError_t launch_distill_targets(const ModelDesc& m, const float* feat, const float4* dirs, const float4* nrm, int P,
+                                   int K, float* vis, float* depth, int num_sms, cudaStream_t s);
 cudaError_t launch_distill_fp32(const ModelDesc& m, const float4* pos, const float4* nrm, int P, int K,
                                 const float4* dirs, const float* brdf_t, const float* vis_t, const float* depth_t,
                                 float* loss, float* g_table, float* g_brdf, float* g_irt, int num_sms, cudaStream_t s);

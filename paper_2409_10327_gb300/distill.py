@@ -5,7 +5,7 @@
 
 Each step draws K stratified whole-sphere directions per point
 (rt_distill_dirs), takes the teacher's heads from its stage kernels (rt_encode,
-rt_decode, rt_trace), accumulates the student's per-head loss gradient
+rt_decode, rt_distill_targets), accumulates the student's per-head loss gradient
 (rt_distill_backward) and applies Adam (rt_adam_step; learning rate 2e-3,
 weight decay 1e-6 on the MLPs), then rebinds the student's parameters.  This
 module only orders those calls and owns the parameter and moment buffers.
@@ -37,7 +37,7 @@ class Distiller:
         dirs = self.student.distill_dirs(P, self.K, ray_offset)
         feat = self.teacher.encode(pos)
         brdf_t = self.teacher.decode(feat)
-        vis_t, depth_t = self.teacher.trace(feat, dirs)
+        vis_t, depth_t = self.teacher.distill_targets(feat, dirs, normal)
         for g in self.grads:
             g.zero_()
         self.loss.zero_()

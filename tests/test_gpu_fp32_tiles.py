@@ -114,3 +114,25 @@ def test_encode_alignment(lib):
     assert lib.LIB.rt_encode(r.ctx, lib._ptr(pos), 77, lib._ptr(buf[1:]), None, None, None) == lib.RT_OK
     torch.cuda.synchronize()
     assert torch.equal(buf[1:].view(77, 10), want)
+
+
+# the distillation's targets are rt_trace's values at the front-facing directions (within the rounding both are allowed
+# above), and zero visibility at the near depth elsewhere; one and several direction units, a point without any
+@pytest.mark.parametrize("P, K", [(1, 1), (7, 31), (3, 256), (2, 700)])
+def test_distill_targets(lib, P, K):
+    cfg = helpers.small_cfg(levels=5)
+    r = helpers.renderer_for(cfg, scenegen.make_scene(cfg, 6, bias_scale=0.3))
+    rng = np.random.default_rng(P + K)
+    unit = lambda a: a / np.linalg.norm(a, axis=-1, keepdims=True)
+    plane = lambda a: torch.from_numpy(np.concatenate([a, np.zeros(a.shape[:-1] + (1,))], -1).astype(np.float32)).cuda()
+    feat = torch.from_numpy(rng.normal(0, 0.2, (P, 10)).astype(np.float32)).cuda()
+    d, n = unit(rng.normal(size=(P, K, 3))), unit(rng.normal(size=(P, 3)))
+    d[0] = unit(d[0] - 3.0 * n[0])                           # all behind point 0
+    dirs, normal = plane(d), plane(n)
+    vis, depth = r.distill_targets(feat, dirs, normal)
+    tv, td = r.trace(feat, dirs)
+    front = (dirs[..., :3].double() * normal[:, None, :3].double()).sum(-1) > 0
+    assert not front[0].any()
+    assert (vis[~front] == 0).all() and (depth[~front] == cfg.near).all()
+    torch.testing.assert_close(vis[front], tv[front], rtol=0, atol=6e-6)
+    torch.testing.assert_close(depth[front], td[front], rtol=0, atol=6e-6)
