@@ -271,7 +271,8 @@ TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic_frame800.txt")
 KERNEL_SOURCES = {
     "bf16": ["render_bf16.cu", "render_bf16_kernel.cuh", "tc_common.cuh", "fast_math.cuh", "mis.cuh", "mbarrier.cuh",
              "device_common.cuh", "rt_internal.h"],
-    "fp32": ["render_fp32.cu", "warp_gemm.cuh", "mis.cuh", "device_common.cuh", "rt_internal.h"],
+    "fp32": ["render_fp32.cu", "tc_split.cuh", "tc_common.cuh", "fast_math.cuh", "mbarrier.cuh", "warp_gemm.cuh", "mis.cuh",
+             "device_common.cuh", "rt_internal.h"],
 }
 
 
@@ -364,6 +365,8 @@ def _roofline(cfg, launch_ms, peaks, probes=None):
         else:
             roof = {"bound": "alu", "achieved": flop / avg_s / 1e12, "peak": FP32_ALU_PEAK_TFLOPS, "unit": "TFLOP/s",
                     "peak_source": "nominal: 152 SMs x 128 FP32 lanes x 2 FLOP x 2.07 GHz"}
+        roof["note"] = ("the M secondary evaluations run on the tensor cores as three-part bf16 products (6 per FP32 product): "
+                        "the FMA rate is a scale, not a ceiling")
     else:
         # one launch of tens of ms timed alone is a burst: the burst cuBLAS figure is its denominator
         pk = peaks.get("bf16_tflops")

@@ -1,5 +1,5 @@
 // Stages (b) and (c) on their own: B at given features (rt_decode) and I at
-// given features and directions (rt_trace; also the distillation's teacher).
+// given features and directions (rt_trace).
 // Rows, (point) or (point, direction) consecutively, run 128 at a time through
 // the tensor-core layers of tc_split.cuh, as in the FP32 frame kernel: a
 // warpgroup per tile, thread = row = TMEM lane, three warpgroups per SM that
