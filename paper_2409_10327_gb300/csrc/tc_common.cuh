@@ -50,7 +50,8 @@ __device__ __forceinline__ uint64_t sdesc32(uint32_t saddr) {
 // Issue.  A whole warp runs a chain's code with one lane elected (`one`, a
 // predicate of each instruction): in a one-thread branch every operand has to
 // be moved to uniform registers first, which for short MMAs (32 cycles each)
-// takes longer than the MMA.
+// takes longer than the MMA: the 800 x 800 x 128 BF16 frame went from 39.3 to
+// 35.7 ms, the FP32 one from 166 to 150.
 __device__ __forceinline__ uint32_t elect_one() {
   uint32_t r;
   asm volatile(
