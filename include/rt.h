@@ -221,7 +221,10 @@ rt_status rt_shade(rt_ctx* ctx, const rt_gbuffer* pts, int64_t P, int32_t level,
 
 /* Stages (a)-(e) fused in one persistent kernel: radiance [P][4] (rgb, 0) of
  * the P G-buffer points; point p uses RNG pixel id pixel_offset + p, so a
- * frame rendered in shards equals the frame rendered at once.
+ * frame rendered in shards, of any sizes, equals the frame rendered at once:
+ * bit for bit on RT_FP32, and on RT_BF16 (soft visibility) for n_dirs a
+ * multiple of 32; for other n_dirs a pixel's directions may be grouped
+ * differently in its BF16 sum, and shards agree up to float rounding.
  * With cfg.visibility = RT_VIS_HARD the BF16 path does the secondary work
  * (x' encode, B, the M secondary I evaluations, Eq. 1 at x') only for shadow
  * directions: each warpgroup queues its shadow rows in shared memory and

@@ -73,6 +73,7 @@ constexpr int SM_WG = WBF16_BYTES;
 static_assert(WG_MISC + 16 + kCarrySlots * 8 * 16 <= WG_BYTES, "warpgroup block overflow");
 static_assert(WG_CNT + 16 <= WG_BYTES_HARD, "warpgroup block overflow (hard visibility)");
 static_assert(64 * 64 <= 2 * kPixSlots * 64, "the replicas' exchanged features fit the slots");
+static_assert(3 * 96 * 3 * 4 <= 2 * kPixSlots * 64, "so do the terms of replicas 1 .. 3");
 static_assert(128 * 16 <= 2 * kPixSlots * 64 && WG_MISC % 16 == 0 && WG_BYTES_HARD % 16 == 0, "pixel slots");
 
 template <int WG, bool HARD = false>
@@ -389,8 +390,9 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
     // constant 0, which keeps the consecutive order's code as tight as without the option)
     // REP > 1 (a launch whose warpgroups have no more than R = 128 / REP samples each): a tile holds R
     // samples, each by REP rows, its replicas.  They share the sample's serial chain: each encodes
-    // 16 / REP levels of x' and takes every REP-th secondary direction, and the partial sums meet at
-    // the end, so the chain is 1 + 1 + M / REP evaluations long instead of 2 + M.
+    // 16 / REP levels of x' and takes every REP-th secondary direction, so the chain is 1 + 1 + M / REP
+    // evaluations long instead of 2 + M.  Replica 0 adds every direction's term in the order of j, as a
+    // row on its own does: the bits of a sample, and so of a shard, do not depend on the launch's size.
     constexpr int R = 128 / REP;
     static_assert(REP == 1 || (!HARD && !CHUNK), "replicas: the consecutive soft order only");
     const int rep = REP > 1 ? t / R : 0, tr = REP > 1 ? t % R : t;
@@ -465,7 +467,7 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
       // this row is fr1 (v Lenv(w_i) + (1 - v) (pi/M) sum_j v'_j fr2_j Lenv(w'_j)).
       f3 c[NL];
       {
-        const f3 w0 = fr1 * (rep == 0 ? v : 0.0f);
+        const f3 w0 = fr1 * v;
         if (NL == 1) {
           c[0] = w0 * le1;
         } else {
@@ -516,8 +518,7 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
       // (c) + (e) at x': M directions about n'
       bool ok = true;
       for (int j0 = 0; j0 < M && ok; j0 += REP) {
-        const int j = REP > 1 ? min(j0 + rep, M - 1) : j0;
-        const bool own = REP == 1 || j0 + rep < M;   // a replica beyond the last direction repeats it with weight 0
+        const int j = REP > 1 ? min(j0 + rep, M - 1) : j0;   // (a replica beyond the last direction: not added below)
         const f3 wj = cosine_direction_fast(n2, m.seed, dir_counter(q, M, 1 + j));
         const EnvTap tapj = env_tap_fast(m.env_h, m.env_w, wj);
         const f3 frw = fr1 * brdf_eval_fast(a2, r2, n2, wj, wo2, m.f0, m.lambert);
@@ -530,8 +531,43 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
         ok = run_mma([&](uint32_t one) { mma_layer2(one, D_t, H_t, W_s + OFFB_IW2, W_s + OFFB_ONES, W_s + OFFB_IB2); });
         if (!ok) break;
         const float v2 = m.force_vis2 >= 0.f ? m.force_vis2 : sigmoid_fast(head_vis(D_w, hp.iw3v, hp.ib3[0]));
-        const f3 wj3 = frw * (own ? wsec * v2 : 0.0f);
-        if (NL == 1) {
+        const f3 wj3 = frw * (wsec * v2);
+        if constexpr (REP > 1) {
+          // The other replicas' weights and, light by light in two buffers, their Lenv(w'_j) through the feature
+          // slots, which B has consumed; the round trips of the next directions come before these are written again.
+          constexpr int kOther = 128 - R;
+          float* xw = reinterpret_cast<float*>(fpix);
+          f3 lights[NL];   // fetched together, before the barriers
+#pragma unroll
+          for (int e = 0; e < NL; ++e) lights[e] = NL == 1 ? lej : env_fetch(envs + e * env_hw, tapj);
+#pragma unroll
+          for (int e = 0; e < NL; ++e) {
+            const f3 le = lights[e];
+            float* xl = xw + 3 * kOther * (1 + (e & 1));
+            if (rep > 0) {
+              const int o = t - R;
+              if (e == 0) {
+                xw[o] = wj3.x;
+                xw[kOther + o] = wj3.y;
+                xw[2 * kOther + o] = wj3.z;
+              }
+              xl[o] = le.x;
+              xl[kOther + o] = le.y;
+              xl[2 * kOther + o] = le.z;
+            }
+            wg_sync(wg);
+            if (rep == 0) {
+              c[e] = c[e] + wj3 * le;
+#pragma unroll
+              for (int k = 1; k < REP; ++k) {
+                if (j0 + k < M) {
+                  const int o = t + R * (k - 1);
+                  c[e] = c[e] + mk(xw[o], xw[kOther + o], xw[2 * kOther + o]) * mk(xl[o], xl[kOther + o], xl[2 * kOther + o]);
+                }
+              }
+            }
+          }
+        } else if (NL == 1) {
           c[0] = c[0] + wj3 * lej;
         } else {
   #pragma unroll
@@ -539,22 +575,6 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
         }
       }
       if (!ok) break;
-
-      if constexpr (REP > 1) {   // the replicas' partial sums into replica 0's rows
-#pragma unroll
-        for (int e = 0; e < NL; ++e) {
-          wg_sync(wg);   // the exchanged features (first light) or the previous light's sums are read
-          red[t] = make_float4(c[e].x, c[e].y, c[e].z, 0.f);
-          wg_sync(wg);
-          if (rep == 0) {
-#pragma unroll
-            for (int k = 1; k < REP; ++k) {
-              const float4 h = red[t + R * k];
-              c[e] = mk(c[e].x + h.x, c[e].y + h.y, c[e].z + h.z);
-            }
-          }
-        }
-      }
 
       // deterministic segmented reduction of the tile's rows into their pixels,
       // one light at a time

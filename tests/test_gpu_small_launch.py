@@ -33,3 +33,26 @@ def test_small_launch_equals_large(n_dirs, m_dirs, sizes, lights):
         np.testing.assert_allclose(got, whole[:, lo:lo + n], rtol=(n_dirs + m_dirs) * 2.0 ** -23, atol=0)
         lo += n
     assert r.check() == 0
+
+
+# a frame above the small-launch rule against shards on both sides of it, one of them by two replicas at 32 directions:
+# with a multiple of 32 directions the pixel sums group alike too, so every bit is the frame's
+@pytest.mark.parametrize("n_dirs, m_dirs, lights, kw", [(32, 8, 1, {}), (32, 5, 8, {}), (32, 1, 3, {}), (64, 8, 2, {}),
+                                                        (64, 3, 1, {"sampling": 1}), (32, 6, 5, {"force_vis2": 0.25})])
+def test_shards_have_the_frames_bits(n_dirs, m_dirs, lights, kw):
+    workers = 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    per = -(-72 // n_dirs)                       # pixels per warpgroup that make more than 64 samples
+    P = 2 * workers * per + 11
+    cfg = helpers.small_cfg(n_dirs=n_dirs, m_dirs=m_dirs, precision="bf16")
+    sc, gb = helpers.scene_arrays(cfg, 7, bias=0.2, n_pixels=P)
+    r = helpers.renderer_for(cfg, sc, **kw)
+    dgb = helpers.to_cuda(gb)
+    envs = torch.from_numpy(np.stack([np.roll(sc.env, 3 * e, axis=1) for e in range(lights)])).cuda()
+    whole = r.render_frame_multi(dgb, envs, pixel_offset=3).cpu().numpy()
+    cuts = [0, 1, 8, 8 + workers // 2, 8 + workers // 2 + (64 // n_dirs) * workers, P]
+    assert cuts[-1] - cuts[-2] > workers * (per - 1)   # the last shard is above the rule, the others below
+    for lo, hi in zip(cuts, cuts[1:]):
+        part = {k: v[lo:hi].contiguous() for k, v in dgb.items()}
+        got = r.render_frame_multi(part, envs, pixel_offset=3 + lo).cpu().numpy()
+        np.testing.assert_array_equal(got, whole[:, lo:hi])
+    assert r.check() == 0
