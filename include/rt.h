@@ -257,13 +257,18 @@ rt_status rt_render_frame_multi(rt_ctx* ctx, const rt_gbuffer* gb, int64_t P, in
  * workload, writing radiance as rt_render_frame_multi does, keeps the fastest
  * in the context and returns its time in *best_ms (may be NULL; -1 for the
  * FP32 path, which has one shape).  Tile shapes that do not divide n_dirs, or
- * RT_VIS_HARD, are skipped.  Synchronises `stream`. */
+ * RT_VIS_HARD, are skipped.  On a workload of few samples (see
+ * rt_set_launch_shape) only the lights per launch are tuned.  Synchronises
+ * `stream`. */
 rt_status rt_tune(rt_ctx* ctx, const rt_gbuffer* gb, int64_t P, int64_t pixel_offset, const float* envs, int32_t E,
                   float* radiance, void* stream, float* best_ms);
 
 /* Read or force the BF16 launch shape (lights_per_launch in {1,2,4,8},
  * warpgroups in {2,3,4}; anything else is RT_ERR_INVALID_ARG).  RT_VIS_HARD
- * renders ignore the warpgroups part (always 4). */
+ * renders ignore the warpgroups part (always 4).  Soft-visibility launches of
+ * few samples, ceil(P / (4 SMs)) n_dirs <= 64, share a sample's work over
+ * several rows of a tile in a kernel of their own and ignore the warpgroups and
+ * the tile shape. */
 rt_status rt_tuned_shape(const rt_ctx* ctx, int32_t* lights_per_launch, int32_t* warpgroups);
 rt_status rt_set_launch_shape(rt_ctx* ctx, int32_t lights_per_launch, int32_t warpgroups);
 

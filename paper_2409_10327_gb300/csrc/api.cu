@@ -479,11 +479,17 @@ rt_status rt_tune(rt_ctx* ctx, const rt_gbuffer* gb, int64_t P, int64_t pixel_of
   int best_nl = ctx->tuned_nl, best_wg = ctx->tuned_wg, best_dpt = ctx->tuned_dpt;
   st = RT_OK;
   const int N = ctx->cfg.n_dirs;
+  // A launch of few samples has one kernel whatever the warpgroups and the tile shape: only the lights per launch are
+  // timed, and the other two stay as they are for the context's larger frames.
+  const bool one_shape = ctx->cfg.visibility != RT_VIS_HARD && small_replicas((int)P, N, ctx->num_sms) > 1;
   for (int dpt = 128; dpt >= 32 && st == RT_OK; dpt /= 2) {
     // a tile of 128 / dpt pixels x dpt directions; other shapes repeat the consecutive order
-    if (dpt < 128 && (ctx->cfg.visibility == RT_VIS_HARD || N % dpt != 0 || N <= dpt)) continue;
+    if (one_shape ? dpt != ctx->tuned_dpt
+                  : dpt < 128 && (ctx->cfg.visibility == RT_VIS_HARD || N % dpt != 0 || N <= dpt))
+      continue;
     m.dpt = dpt;
     for (int wg = ctx->cfg.visibility == RT_VIS_HARD ? 4 : 2; wg <= 4 && st == RT_OK; ++wg) {
+      if (one_shape && wg != ctx->tuned_wg) continue;
       for (int nl = 1; nl <= 8 && st == RT_OK; nl *= 2) {
         if (nl > 1 && nl / 2 >= E) break;   // wider launches than E lights repeat the previous shape
         float ms = 0.0f;

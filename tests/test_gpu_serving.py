@@ -149,3 +149,18 @@ def test_tile_shapes_give_the_same_bits(lib, n_dirs, P):
         with pytest.raises(lib.RtError) as e:
             r.set_tile_shape(bad)
         assert e.value.status == lib.RT_ERR_INVALID_ARG
+
+
+def test_tuner_keeps_the_shape_on_small_launches(lib):
+    # one kernel serves such a launch whatever its warpgroups and tile shape, so timing cannot choose them
+    cfg = helpers.small_cfg(n_dirs=64, m_dirs=2, precision="bf16")
+    sc = scenegen.make_scene(cfg, 1)
+    gb = helpers.to_cuda(scenegen.make_gbuffer(100, 6))
+    denv = torch.from_numpy(_envs(cfg, 2)).cuda()
+    r = helpers.renderer_for(cfg, sc)
+    for wg in (2, 3, 4):
+        for dpt in (128, 64, 32):
+            r.set_launch_shape(8, wg)
+            r.set_tile_shape(dpt)
+            assert r.tune(gb, denv) > 0
+            assert r.launch_shape()[1] == wg and r.tile_shape() == dpt and r.launch_shape()[0] in (1, 2)
