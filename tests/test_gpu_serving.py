@@ -151,6 +151,12 @@ def test_tile_shapes_give_the_same_bits(lib, n_dirs, P):
         assert e.value.status == lib.RT_ERR_INVALID_ARG
 
 
+def _above_small(n_dirs, fill=1.0):
+    """Points that give each of the chip's warpgroups more than the 64 samples of a small launch."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return int(4 * sms * -(-72 // n_dirs) * fill)
+
+
 def test_tuner_keeps_the_shape_on_small_launches(lib):
     # one kernel serves such a launch whatever its warpgroups and tile shape, so timing cannot choose them
     cfg = helpers.small_cfg(n_dirs=64, m_dirs=2, precision="bf16")
@@ -164,3 +170,47 @@ def test_tuner_keeps_the_shape_on_small_launches(lib):
             r.set_tile_shape(dpt)
             assert r.tune(gb, denv) > 0
             assert r.launch_shape()[1] == wg and r.tile_shape() == dpt and r.launch_shape()[0] in (1, 2)
+
+
+# every launch and tile shape on frames above the small-launch rule (below it they are one kernel): with a multiple of 32
+# directions the bits do not depend on warpgroups and tile shape
+@pytest.mark.parametrize("n_dirs, m_dirs", [(64, 2), (32, 3), (128, 1)])
+def test_launch_shapes_give_the_same_bits(lib, n_dirs, m_dirs):
+    cfg = helpers.small_cfg(n_dirs=n_dirs, m_dirs=m_dirs, precision="bf16")
+    sc = scenegen.make_scene(cfg, 3, bias_scale=0.1)
+    P = _above_small(n_dirs) + 17
+    gb = helpers.to_cuda(scenegen.make_gbuffer(P, 8))
+    envs = _envs(cfg, 5)
+    denv = torch.from_numpy(envs).cuda()
+    r = helpers.renderer_for(cfg, sc)
+    want = np.stack([_single_light(cfg, sc, gb, e, 7, (1, 4)) for e in envs])
+    for nl in (1, 2, 4, 8):
+        first = None
+        for wg in (4, 3, 2):
+            for dpt in (128, 64, 32):
+                r.set_tile_shape(dpt)
+                r.set_launch_shape(nl, wg)
+                got = r.render_frame_multi(gb, denv, pixel_offset=7).cpu().numpy()
+                first = got if first is None else first
+                np.testing.assert_array_equal(got, first, err_msg=str((nl, wg, dpt)))
+        assert helpers.rel_err(first[..., :3], want[..., :3]) <= 1e-5, nl
+    assert r.check() == 0
+
+
+# the same shapes at direction counts whose pixels start anywhere in a tile, where the grouping of a sum may differ
+@pytest.mark.parametrize("n_dirs", [48, 4, 33])
+def test_multi_light_shapes_above_the_small_rule(lib, n_dirs):
+    cfg = helpers.small_cfg(n_dirs=n_dirs, m_dirs=4, precision="bf16")
+    sc = scenegen.make_scene(cfg, 0, bias_scale=0.1)
+    gb = helpers.to_cuda(scenegen.make_gbuffer(_above_small(n_dirs, 1.3), 5))
+    envs = _envs(cfg, 5)
+    denv = torch.from_numpy(envs).cuda()
+    r = helpers.renderer_for(cfg, sc)
+    for shape in [(nl, wg) for nl in (1, 2, 4, 8) for wg in (2, 3, 4)]:
+        r.set_launch_shape(*shape)
+        out = r.render_frame_multi(gb, denv, pixel_offset=7).cpu().numpy()
+        for e in (0, 4):
+            ref = _single_light(cfg, sc, gb, envs[e], 7, (1, 4))
+            # sums of the same non-negative terms in another grouping: N + M roundings of 2^-24 on either side
+            np.testing.assert_allclose(out[e, :, :3], ref[:, :3], rtol=(n_dirs + 4) * 2.0 ** -23, atol=0, err_msg=str(shape))
+            assert np.all(out[e, :, 3] == 0)
