@@ -174,7 +174,12 @@ rt_status rt_set_params(rt_ctx* ctx, const void* table, const float* brdf_w, con
                         const float* env, void* stream);
 
 /* Read (and clear) the device status word written by bounded waits and
- * bounds checks; synchronises `stream`.  *word = 0 when nothing fired. */
+ * bounds checks; synchronises `stream`.  *word = 0 when nothing fired.  Every
+ * kernel that issues tensor-core work has such waits (rt_decode, rt_trace, the
+ * frames of both precisions, the BF16 rt_backward): a wait that runs out (2 s)
+ * ends a part of the launch, whose outputs are then unspecified, and sets
+ * (1 << 28) | a bit for the kernel: 1 BF16 frame, 2 BF16 adjoint, 4 rt_decode
+ * or rt_trace, 8 FP32 frame.  Returns RT_ERR_TIMEOUT then. */
 rt_status rt_check(rt_ctx* ctx, uint32_t* word, void* stream);
 
 /* ---- stages ------------------------------------------------------------- */
@@ -329,14 +334,20 @@ rt_status rt_backward(rt_ctx* ctx, const rt_gbuffer* gb, int64_t P, int64_t pixe
  *  - all calls on a device share the array: calls whose work overlaps on the
  *    GPU (different streams, or different models in flight) race; serialise
  *    them on one stream;
- *  - no cudaMalloc, cudaFree or allocating library routine is called.
+ *  - no cudaMalloc, cudaFree or allocating library routine is called;
+ *  - a bounded wait that runs out is recorded in a status word beside the
+ *    array, one per device: rt_check_static reads it.
  * Results equal rt_render_frame's for the same inputs. */
 rt_status rt_render_frame_static(const rt_config* cfg, const void* table, const float* brdf_w, const float* irt_w,
                                  const float* env, const rt_gbuffer* gb, int64_t P, int64_t pixel_offset,
                                  float* radiance, void* stream);
 
+/* rt_check for rt_render_frame_static: read and clear the current device's
+ * status word; synchronises `stream`.  The set-up of a first call, as above. */
+rt_status rt_check_static(uint32_t* word, void* stream);
+
 /* ---- fault-path self-tests ------------------------------------------------
- * The paper has no counterpart: these two calls let a test drive the
+ * The paper has no counterpart: these calls let a test drive the
  * library's own failure handling without faulting or hanging a GPU. */
 
 /* Run the device-side timeout path of the tensor-core kernels: one warp
@@ -346,6 +357,9 @@ rt_status rt_render_frame_static(const rt_config* cfg, const void* table, const 
  * following rt_check returns RT_ERR_TIMEOUT with word = (1 << 28) | 0xF.
  * Needs a context (rt_set_params not required); asynchronous on `stream`. */
 rt_status rt_selftest_wait(rt_ctx* ctx, int64_t limit_ns, void* stream);
+
+/* The same on the status word of rt_render_frame_static (rt_check_static). */
+rt_status rt_selftest_wait_static(int64_t limit_ns, void* stream);
 
 /* Host-side fault injection for rt_create: the n-th device allocation that
  * rt_create makes from now on fails as if cudaMalloc had reported an

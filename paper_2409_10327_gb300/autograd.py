@@ -5,7 +5,9 @@
 The forward binds the parameters (rt_set_params) and runs the fused kernel;
 the backward calls the hand-written adjoint kernel, which recomputes the
 activations and accumulates gradients for the hash table and both packed MLP
-blobs.  Sampled directions are constants of the estimator.
+blobs.  Sampled directions are constants of the estimator.  Neither call
+synchronises for the status word: renderer.check() says whether a bounded wait
+of either ran out.
 """
 from __future__ import annotations
 

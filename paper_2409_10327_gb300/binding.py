@@ -31,7 +31,8 @@ EXPORTS = ["rt_status_str", "rt_config_default", "rt_config_validate", "rt_level
            "rt_render_frame", "rt_backward", "rt_render_frame_static", "rt_render_frame_multi", "rt_tune",
            "rt_tuned_shape", "rt_set_launch_shape", "rt_tuned_tile_shape", "rt_set_tile_shape", "rt_denoise", "rt_distill_dirs",
            "rt_distill_targets",
-           "rt_distill_backward", "rt_adam_step", "rt_selftest_wait", "rt_debug_fail_alloc",
+           "rt_distill_backward", "rt_adam_step", "rt_selftest_wait", "rt_check_static",
+           "rt_selftest_wait_static", "rt_debug_fail_alloc",
            "rt_probe_gather", "rt_probe_ffma"]
 
 
@@ -95,6 +96,8 @@ def _load() -> ctypes.CDLL:
         "rt_distill_backward": (I32, [P, P, P, I64, I32, P, P, P, P, P, P, P, P, P]),
         "rt_adam_step": (I32, [P, P, P, P, I64, F32, F32, F32, F32, F32, I32, P]),
         "rt_selftest_wait": (I32, [P, I64, P]),
+        "rt_check_static": (I32, [ctypes.POINTER(ctypes.c_uint32), P]),
+        "rt_selftest_wait_static": (I32, [I64, P]),
         "rt_debug_fail_alloc": (I32, [I32]),
         "rt_probe_gather": (I32, [P, I64, I32, I32, I32, P, P]),
         "rt_probe_ffma": (I32, [I32, I32, P, P]),

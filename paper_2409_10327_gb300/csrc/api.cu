@@ -131,6 +131,16 @@ bool check_gbuffer(const rt_gbuffer* gb) {
 
 }  // namespace
 
+rt_status rtk::read_status(uint32_t* status, uint32_t* word, cudaStream_t s) {
+  uint32_t h = 0;
+  if (cudaMemcpyAsync(&h, status, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess) return RT_ERR_CUDA;
+  if (cudaStreamSynchronize(s) != cudaSuccess) return RT_ERR_CUDA;
+  if (cudaMemsetAsync(status, 0, 4, s) != cudaSuccess) return RT_ERR_CUDA;
+  *word = h;
+  if (h == 0) return RT_OK;
+  return (h >> 28) == 1 ? RT_ERR_TIMEOUT : RT_ERR_BOUNDS;
+}
+
 extern "C" {
 
 const char* rt_status_str(rt_status s) {
@@ -324,8 +334,7 @@ rt_status rt_set_params(rt_ctx* ctx, const void* table, const float* brdf_w, con
 
 rt_status rt_selftest_wait(rt_ctx* ctx, int64_t limit_ns, void* stream) {
   if (ctx == nullptr) return RT_ERR_INVALID_ARG;
-  const int64_t lim = limit_ns < 1000000 ? 1000000 : (limit_ns > 2000000000 ? 2000000000 : limit_ns);
-  return cuda_status(launch_wait_never(ctx->status, (uint64_t)lim, (cudaStream_t)stream));
+  return cuda_status(launch_wait_never(ctx->status, limit_ns, (cudaStream_t)stream));
 }
 
 rt_status rt_debug_fail_alloc(int32_t n) {
@@ -336,14 +345,7 @@ rt_status rt_debug_fail_alloc(int32_t n) {
 
 rt_status rt_check(rt_ctx* ctx, uint32_t* word, void* stream) {
   if (ctx == nullptr || word == nullptr) return RT_ERR_INVALID_ARG;
-  cudaStream_t s = (cudaStream_t)stream;
-  uint32_t h = 0;
-  if (cudaMemcpyAsync(&h, ctx->status, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess) return RT_ERR_CUDA;
-  if (cudaStreamSynchronize(s) != cudaSuccess) return RT_ERR_CUDA;
-  if (cudaMemsetAsync(ctx->status, 0, 4, s) != cudaSuccess) return RT_ERR_CUDA;
-  *word = h;
-  if (h == 0) return RT_OK;
-  return (h >> 28) == 1 ? RT_ERR_TIMEOUT : RT_ERR_BOUNDS;
+  return read_status(ctx->status, word, (cudaStream_t)stream);
 }
 
 rt_status rt_encode(rt_ctx* ctx, const float* pos, int64_t P, float* feat, uint32_t* idx, float* w, void* stream) {

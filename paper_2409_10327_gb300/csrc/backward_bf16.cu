@@ -36,7 +36,7 @@
 // own slice of a staging tile (free once the MMAs that read it completed) and
 // adds to the caller's blob with coalesced global reductions (float4 where the
 // blobs are 16-byte aligned).  Every mbarrier wait is bounded; on expiry the
-// warpgroup records kStatusTimeout | 2 and stops.
+// warpgroup records kStatusTimeout | kWhereBackwardBf16 and stops.
 #include "adjoint.cuh"
 #include "mbarrier.cuh"
 #include "mis.cuh"
@@ -283,7 +283,7 @@ backward_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant_
       __syncwarp();
     }
     if (!mbar_wait(bar_a, phase)) {
-      if (!abort && t == 0) atomicOr(m.status, kStatusTimeout | 2u);
+      if (!abort && t == 0) atomicOr(m.status, kStatusTimeout | kWhereBackwardBf16);
       abort = 1;
       pending_phase = phase;
     }

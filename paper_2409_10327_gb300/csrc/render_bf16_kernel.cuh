@@ -164,7 +164,7 @@ render_bf16_kernel(const __grid_constant__ ModelDesc m, const __grid_constant__ 
       __syncwarp();
     }
     if (!mbar_wait(bar_a, phase)) {
-      if (!abort && t == 0) atomicOr(m.status, kStatusTimeout | 1u);
+      if (!abort && t == 0) atomicOr(m.status, kStatusTimeout | kWhereRenderBf16);
       abort = 1;
       pending_phase = phase;
     }

@@ -219,7 +219,7 @@ render_fp32_kernel(const __grid_constant__ ModelDesc m, rt_gbuffer gb, int P, lo
   };
   auto wait = [&] {
     if (!mbar_wait(bar, phase)) {
-      if (!abort && t == 0 && m.status != nullptr) atomicOr(m.status, kStatusTimeout | 2u);
+      if (!abort && t == 0) atomicOr(m.status, kStatusTimeout | kWhereRenderFp32);
       abort = 1;
       pending_phase = phase;
     }

@@ -146,10 +146,17 @@ cudaError_t launch_render_bf16_small(int rep, int nl, const ModelDesc& m, const 
 cudaError_t launch_render_bf16_lights(const ModelDesc& m, const HeadParams& hp, const rt_gbuffer& gb, int P,
                                       long long offset, const float4* envs, int E, float4* out, int num_sms,
                                       int max_nl, int wg, cudaStream_t s);
-// Status-word codes: (kStatusTimeout | where) after a bounded wait gave up.
+// Status-word codes: (kStatusTimeout | where) after a bounded wait gave up, a bit per kernel (words are ORed).
 constexpr uint32_t kStatusTimeout = 1u << 28;
+constexpr uint32_t kWhereRenderBf16 = 1u;
+constexpr uint32_t kWhereBackwardBf16 = 2u;
+constexpr uint32_t kWhereStageMlp = 4u;     // rt_decode, rt_trace
+constexpr uint32_t kWhereRenderFp32 = 8u;
 constexpr uint32_t kWhereSelftest = 0xFu;   // the wait of rt_selftest_wait
-cudaError_t launch_wait_never(uint32_t* status, uint64_t limit_ns, cudaStream_t s);
+// Read and clear a status word (rt_check's work); synchronises s.
+rt_status read_status(uint32_t* status, uint32_t* word, cudaStream_t s);
+// limit_ns clamped to 1 ms .. 2 s
+cudaError_t launch_wait_never(uint32_t* status, int64_t limit_ns, cudaStream_t s);
 cudaError_t launch_render_fp32(const ModelDesc& m, const rt_gbuffer& gb, int P, long long offset,
                                float4* out, int num_sms, cudaStream_t s);
 cudaError_t prepare_distill();

@@ -1,8 +1,8 @@
 // Fault-path self-test of the device-side timeout: one warp waits, with the
 // bounded mbarrier wait of the tensor-core kernels (mbarrier.cuh), on a
 // barrier that nothing ever arrives on.  The wait runs out after its limit,
-// the warp records a timeout code in the context's status word and the kernel
-// returns, so the context stays usable.  Nothing here faults or hangs a GPU.
+// the warp records a timeout code in the status word (the context's, or the
+// static renderer's) and the kernel returns, so the context stays usable.  Nothing here faults or hangs a GPU.
 #include "mbarrier.cuh"
 #include "rt_internal.h"
 
@@ -25,8 +25,9 @@ __global__ void __launch_bounds__(32) wait_never_kernel(uint32_t* status, uint64
 
 }  // namespace
 
-cudaError_t launch_wait_never(uint32_t* status, uint64_t limit_ns, cudaStream_t s) {
-  wait_never_kernel<<<1, 32, 0, s>>>(status, limit_ns);
+cudaError_t launch_wait_never(uint32_t* status, int64_t limit_ns, cudaStream_t s) {
+  const int64_t lim = limit_ns < 1000000 ? 1000000 : (limit_ns > 2000000000 ? 2000000000 : limit_ns);
+  wait_never_kernel<<<1, 32, 0, s>>>(status, (uint64_t)lim);
   return cudaGetLastError();
 }
 

@@ -102,7 +102,7 @@ mlp_rows_kernel(const __grid_constant__ ModelDesc m, const float* __restrict__ f
   };
   auto wait = [&] {
     if (!mbar_wait(bar, phase)) {
-      if (!abort && t == 0) atomicOr(m.status, kStatusTimeout | 3u);
+      if (!abort && t == 0) atomicOr(m.status, kStatusTimeout | kWhereStageMlp);
       abort = 1;
       pending_phase = phase;
     }

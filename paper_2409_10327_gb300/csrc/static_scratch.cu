@@ -9,7 +9,8 @@
 // of the fused kernel; this entry point keeps that workspace in a file-scope
 // __device__ array instead, so the caller only passes its own inputs and
 // output.  Every GPU that loads this library holds the array (61 KB) until
-// the process exits.
+// the process exits, and beside it the status word in which the kernel records
+// a bounded wait that ran out (rt_check_static reads it).
 #include <mutex>
 
 #include "rt_internal.h"
@@ -18,6 +19,7 @@ namespace rtk {
 
 // The packed FP32 weight image of rt_internal.h, shared by every call.
 static __device__ __align__(256) float g_static_wpack[WPACK_FLOATS];
+static __device__ uint32_t g_static_status;
 
 cudaError_t prepare_render_fp32();
 
@@ -28,6 +30,7 @@ constexpr int kMaxDevices = 64;
 struct DeviceSlot {
   bool ready = false;
   float* wpack = nullptr;   // device address of g_static_wpack on this device
+  uint32_t* status = nullptr;   // and of g_static_status
   int num_sms = 0;
 };
 
@@ -45,15 +48,17 @@ rt_status device_slot(DeviceSlot** out) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return RT_ERR_CUDA;
   if (dev >= kMaxDevices) return RT_ERR_UNSUPPORTED;
-  void* p = nullptr;
+  void *p = nullptr, *w = nullptr;
   if (cudaGetSymbolAddress(&p, g_static_wpack) != cudaSuccess || p == nullptr) return RT_ERR_CUDA;
+  if (cudaGetSymbolAddress(&w, g_static_status) != cudaSuccess || w == nullptr) return RT_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_mutex);
   DeviceSlot& s = g_slots[dev];
-  if (!s.ready || s.wpack != static_cast<float*>(p)) {
+  if (!s.ready || s.wpack != static_cast<float*>(p) || s.status != static_cast<uint32_t*>(w)) {
     s.ready = false;
     if (cudaDeviceGetAttribute(&s.num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return RT_ERR_CUDA;
     if (prepare_render_fp32() != cudaSuccess) return RT_ERR_CUDA;
     s.wpack = static_cast<float*>(p);
+    s.status = static_cast<uint32_t*>(w);
     s.ready = true;
   }
   *out = &s;
@@ -100,6 +105,7 @@ extern "C" rt_status rt_render_frame_static(const rt_config* cfg, const void* ta
     m.grid.dense[l] = l < cfg->levels ? rt_level_is_dense(cfg, l) : 0;
   }
   m.wpack = slot->wpack;
+  m.status = slot->status;
   m.env = reinterpret_cast<const float4*>(env);
   m.env_h = cfg->env_h;
   m.env_w = cfg->env_w;
@@ -124,4 +130,18 @@ extern "C" rt_status rt_render_frame_static(const rt_config* cfg, const void* ta
       cudaSuccess)
     return RT_ERR_CUDA;
   return RT_OK;
+}
+
+extern "C" rt_status rt_check_static(uint32_t* word, void* stream) {
+  if (word == nullptr) return RT_ERR_INVALID_ARG;
+  DeviceSlot* slot = nullptr;
+  const rt_status st = device_slot(&slot);
+  return st != RT_OK ? st : read_status(slot->status, word, static_cast<cudaStream_t>(stream));
+}
+
+extern "C" rt_status rt_selftest_wait_static(int64_t limit_ns, void* stream) {
+  DeviceSlot* slot = nullptr;
+  const rt_status st = device_slot(&slot);
+  if (st != RT_OK) return st;
+  return launch_wait_never(slot->status, limit_ns, static_cast<cudaStream_t>(stream)) == cudaSuccess ? RT_OK : RT_ERR_CUDA;
 }

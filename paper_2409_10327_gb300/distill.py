@@ -8,7 +8,8 @@ Each step draws K stratified whole-sphere directions per point
 rt_decode, rt_distill_targets), accumulates the student's per-head loss gradient
 (rt_distill_backward) and applies Adam (rt_adam_step; learning rate 2e-3,
 weight decay 1e-6 on the MLPs), then rebinds the student's parameters.  This
-module only orders those calls and owns the parameter and moment buffers.
+module only orders those calls and owns the parameter and moment buffers;
+teacher.check() says whether a bounded wait of the teacher's decode ran out.
 """
 from __future__ import annotations
 

@@ -5,7 +5,8 @@ environment maps on a shared geometry pass); the V calls are captured once
 into a CUDA graph and replayed as a single launch.  Timing events recorded
 between the views inside the graph give per-view latencies.  Before capture
 the context's launch shape can be picked by the native autotuner (rt_tune) on
-the first view (or a slice of it).
+the first view (or a slice of it).  A replay does not synchronise for the
+status word: renderer.check() says whether a bounded wait ran out.
 """
 from __future__ import annotations
 

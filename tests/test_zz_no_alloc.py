@@ -99,3 +99,19 @@ def test_static_entry_rejects_what_it_cannot_hold(lib):
     assert call(lib.make_config(cfg, levels=17)) == lib.RT_ERR_INVALID_ARG
     ok = lib.make_config(cfg)
     assert lib.LIB.rt_render_frame_static(ctypes.byref(ok), null, null, null, null, None, 0, 0, null, null) == lib.RT_OK
+
+
+def test_static_entry_reports_a_wait_that_ran_out(lib):
+    # the same word that the static frame's waits write, by a wait on a barrier that nothing arrives on
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    word = ctypes.c_uint32(7)
+    assert lib.LIB.rt_check_static(ctypes.byref(word), stream) == lib.RT_OK and word.value == 0
+    assert lib.LIB.rt_selftest_wait_static(20_000_000, stream) == lib.RT_OK
+    assert lib.LIB.rt_check_static(ctypes.byref(word), stream) == lib.RT_ERR_TIMEOUT
+    assert word.value == (1 << 28) | 0xF
+    cfg = helpers.small_cfg()
+    sc = scenegen.make_scene(cfg, 0)
+    out = _static_render(lib, lib.make_config(cfg), sc, helpers.to_cuda(scenegen.make_gbuffer(33, 4)))
+    assert np.isfinite(out).all()
+    assert lib.LIB.rt_check_static(ctypes.byref(word), stream) == lib.RT_OK and word.value == 0
+    assert lib.LIB.rt_check_static(None, stream) == lib.RT_ERR_INVALID_ARG
