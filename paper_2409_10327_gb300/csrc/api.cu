@@ -24,6 +24,7 @@ struct rt_ctx {
   const void* table;
   const float* env;
   HeadParams head;     // host copy of the FP32 output layers (BF16 kernel parameter)
+  int done_slot;       // the count (kDoneWord + 0 or 1) of the next rt_set_params; the other one is cleared by it
   bool ready;
   int tuned_nl;        // lights per launch of the BF16 kernel (rt_tune), default 8
   int tuned_wg;        // warpgroups per CTA of the BF16 kernel (rt_tune), default 4
@@ -33,7 +34,7 @@ struct rt_ctx {
 namespace {
 
 constexpr int64_t kMaxP = 2147483647LL;
-constexpr int kDoneWord = 32;   // words 32 and 33 of the status block: rt_set_params' count of finished rows
+constexpr int kDoneWord = 32;   // words 32 and 33 of the status block: rt_set_params' counts of finished rows
 
 bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
@@ -255,9 +256,12 @@ rt_status rt_create(const rt_config* cfg, rt_ctx** out) {
     delete ctx;
     return RT_ERR_OOM;
   }
-  if (ws_malloc((void**)&ctx->status, 256) != cudaSuccess || cudaMemset(ctx->status, 0, 256) != cudaSuccess) {
+  // the memset is queued on the legacy stream: it has to be done before a call on any other stream counts in the block
+  if (ws_malloc((void**)&ctx->status, 256) != cudaSuccess || cudaMemset(ctx->status, 0, 256) != cudaSuccess ||
+      cudaStreamSynchronize(nullptr) != cudaSuccess) {
     cudaFree(ctx->wpack);
     cudaFree(ctx->wbf16);
+    cudaFree(ctx->status);
     delete ctx;
     return RT_ERR_OOM;
   }
@@ -307,7 +311,7 @@ rt_status rt_set_params(rt_ctx* ctx, const void* table, const float* brdf_w, con
       brdf_w, irt_w, lf, ctx->wpack, ctx->wbf16, reinterpret_cast<const float4*>(env), ctx->cfg.env_h, ctx->cfg.env_w,
       ctx->cdf, ctx->cdf + (ctx->cfg.env_h + 1), guide_m_of(ctx->cdf, ctx->cfg), guide_shift(ctx->cfg.env_h),
       guide_c_of(ctx->cdf, ctx->cfg), guide_shift(ctx->cfg.env_w),
-      reinterpret_cast<unsigned long long*>(ctx->status + kDoneWord), s));
+      ctx->status + kDoneWord + ctx->done_slot, ctx->status + kDoneWord + (ctx->done_slot ^ 1), s));
   if (st != RT_OK) return st;
   // Host copy of the output layers for the BF16 kernel's parameters: the two spans of the packed image that hold
   // them (I's W3 and b3; B's W3 and b3) as two rows of one strided copy, 4 KB instead of the image's 61.
@@ -318,6 +322,7 @@ rt_status rt_set_params(rt_ctx* ctx, const void* table, const float* brdf_w, con
                         cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return RT_ERR_CUDA;
+  ctx->done_slot ^= 1;   // the launch has run (under capture it would not have): the other count is clear
   HeadParams& h = ctx->head;
   for (int i = 0; i < 64; ++i) {
     h.iw3[i][0] = host[0][2 * i];

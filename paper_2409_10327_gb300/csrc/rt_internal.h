@@ -168,10 +168,11 @@ cudaError_t launch_distill_fp32(const ModelDesc& m, const float4* pos, const flo
                                 float* loss, float* g_table, float* g_brdf, float* g_irt, int num_sms, cudaStream_t s);
 cudaError_t launch_adam(float* p, const float* g, float* m1, float* m2, long long n, float lr, float b1, float b2,
                         float eps, float wd, float bc1, float bc2, int num_sms, cudaStream_t s);
-// both weight images and the texel CDFs of the map; done: a device counter of finished rows, zero at first
+// both weight images and the texel CDFs of the map; done: a device counter of finished rows, zero before the launch;
+// done_next: another, which the launch sets to zero for the next call
 cudaError_t launch_set_params(const float* brdf_w, const float* irt_w, int lf, float* wpack, uint8_t* wbf16,
                               const float4* env, int H, int W, float* cdf_m, float* cdf_c, int* guide_m, int gm_shift,
-                              int* guide_c, int gc_shift, unsigned long long* done, cudaStream_t s);
+                              int* guide_c, int gc_shift, uint32_t* done, uint32_t* done_next, cudaStream_t s);
 // smallest s with 2^s >= n (n >= 1): the cutpoint tables have 2^s entries
 inline int guide_shift(int n) {
   int s = 0;

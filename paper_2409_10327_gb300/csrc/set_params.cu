@@ -87,13 +87,14 @@ __device__ __forceinline__ void finish_cdf(float* v, int n, float* __restrict__ 
 }
 
 // CTA r < H: the conditional CDF of row r, its cutpoints, and the row's total into cdf_m[r + 1]; the CTA that finishes
-// last (every H-th count of *done, which only grows) turns the totals into the marginal CDF and answers its cutpoints.
+// last (the H-th count of *done, zero before the launch) turns the totals into the marginal CDF and answers its cutpoints.
+// *done_next, the next call's count, is cleared here: no count outlives one call.
 // Further CTAs: kCdfThreads elements of the FP32 image each, then of the BF16 image.
 __global__ void __launch_bounds__(kCdfThreads)
 set_params_kernel(const float* __restrict__ bw, const float* __restrict__ iw, int lf, float* __restrict__ wpack,
                   uint8_t* __restrict__ wbf16, const float4* __restrict__ env, int H, int W, float* cdf_m,
                   float* __restrict__ cdf_c, int* __restrict__ guide_m, int gm_shift, int* __restrict__ guide_c,
-                  int gc_shift, unsigned long long* done) {
+                  int gc_shift, uint32_t* done, uint32_t* done_next) {
   extern __shared__ float4 cdf_smem4[];
   float* v = reinterpret_cast<float*>(cdf_smem4);
   const int r = blockIdx.x;
@@ -120,7 +121,8 @@ set_params_kernel(const float* __restrict__ bw, const float* __restrict__ iw, in
     running_sum(v, W);
     __stcg(cdf_m + r + 1, v[W - 1]);   // turned into the marginal CDF by the last CTA
     __threadfence();
-    last = (atomicAdd(done, 1ull) + 1ull) % (unsigned)H == 0;
+    last = atomicAdd(done, 1u) + 1u == (uint32_t)H;
+    if (r == 0) *done_next = 0u;
   }
   __syncthreads();
   finish_cdf(v, W, cdf_c + (size_t)r * (W + 1), guide_c + ((size_t)r << gc_shift), gc_shift);
@@ -138,11 +140,11 @@ set_params_kernel(const float* __restrict__ bw, const float* __restrict__ iw, in
 
 cudaError_t launch_set_params(const float* brdf_w, const float* irt_w, int lf, float* wpack, uint8_t* wbf16,
                               const float4* env, int H, int W, float* cdf_m, float* cdf_c, int* guide_m, int gm_shift,
-                              int* guide_c, int gc_shift, unsigned long long* done, cudaStream_t s) {
+                              int* guide_c, int gc_shift, uint32_t* done, uint32_t* done_next, cudaStream_t s) {
   // a row or column of at most 8192 floats fits the 48 KB of shared memory that need no opt-in
   const size_t smem = ((size_t)(H > W ? H : W) + 3) / 4 * 16;
   set_params_kernel<<<H + kPackBlocks + kBf16Blocks, kCdfThreads, smem, s>>>(
-      brdf_w, irt_w, lf, wpack, wbf16, env, H, W, cdf_m, cdf_c, guide_m, gm_shift, guide_c, gc_shift, done);
+      brdf_w, irt_w, lf, wpack, wbf16, env, H, W, cdf_m, cdf_c, guide_m, gm_shift, guide_c, gc_shift, done, done_next);
   return cudaGetLastError();
 }
 
