@@ -79,14 +79,16 @@ __device__ __forceinline__ void edge_weights(float (&a)[D], const float (&c)[D],
 
 // The depth term's divisors as factors, log2(e) / (sigma_z |g . s| + eps), for the
 // offsets of a (2R + 1)^2 window: entry (dy + R) * (2R + 1) + dx + R; opposite
-// offsets share one, so only the window's first half is computed.
+// offsets share one, so only the window's first half is computed.  Both sides
+// of the fast division are a quarter of that: it answers 0 for a divisor of
+// 2^126 or more, which a background at the largest depths gives.
 template <int R>
 __device__ __forceinline__ void depth_divisors(float2 g, float step, float sigma_z, float (&inv)[(2 * R + 1) * (2 * R + 1)]) {
   constexpr int D = 2 * R + 1;
 #pragma unroll
   for (int k = 0; k <= D * D / 2; ++k) {
     const float sx = step * (float)(k % D - R), sy = step * (float)(k / D - R);
-    inv[k] = __fdividef(kLog2e, fmaf(sigma_z, fabsf(g.x * sx + g.y * sy), kEps));
+    inv[k] = __fdividef(0.25f * kLog2e, fmaf(0.25f * sigma_z, fabsf(g.x * sx + g.y * sy), 0.25f * kEps));
     inv[D * D - 1 - k] = inv[k];
   }
 }

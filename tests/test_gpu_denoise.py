@@ -114,3 +114,12 @@ def test_denoised_render(lib):
     c = rad.cpu().numpy()[:, :3].reshape(64, 64, 3)
     ref_c, ref_v = oden.svgf(c, z.reshape(64, 64), gb["normal"][:, :3].reshape(64, 64, 3), iterations=3)
     _check(out.reshape(64, 64, 4), ref_c, ref_v)
+
+
+def test_denoise_background_at_a_huge_depth(lib):
+    # the gradient at the silhouette times an offset passes 2^126 (and stays below the largest float)
+    c, z, n = _image(20, 24, 2)
+    z[:, 11:] = 9e37
+    got = _run(lib, c, z, n, iterations=1)
+    ref_c, ref_v = oden.svgf(c, z, n, iterations=1)
+    _check(got, ref_c, ref_v)
