@@ -42,6 +42,9 @@ __device__ __forceinline__ float2 depth_gradient(const float* __restrict__ z, in
   return make_float2(gx, gy);
 }
 
+// sigma_n in units of log2(e); the largest exponents stay finite (times L = 0 they have to give 0)
+__device__ __forceinline__ float normal_exponent(float sigma_n) { return fminf(sigma_n * kLog2e, 3.402823466e38f); }
+
 // -ln(c) for c = n . n' by the series of d = 1 - c (exact for c in [1/2, 2]), d + d^2/2 + ... + d^9/9.  For |d| < 1/8,
 // which neighbouring taps of a smooth surface have, the remainder is below 2^-28 of the sum.
 __device__ __forceinline__ float neg_ln_series(float d) {
@@ -102,7 +105,7 @@ __device__ __forceinline__ void variance_pixel(int W, int H, int x, int y, const
   const f3 np_ = xyz(__ldg(nrm + p));
   float inv[49];
   depth_divisors<3>(depth_gradient(z, W, H, x, y), 1.0f, sigma_z, inv);
-  const float sn = sigma_n * kLog2e;
+  const float sn = normal_exponent(sigma_n);
   float s0 = 0.f, s1 = 0.f, s2 = 0.f;
 #pragma unroll
   for (int dy = -3; dy <= 3; ++dy) {
@@ -175,7 +178,7 @@ __device__ __forceinline__ void atrous_pixel(int W, int H, int step, int x, int 
   float inv[25];
   depth_divisors<2>(depth_gradient(z, W, H, x, y), (float)step, sigma_z, inv);
   constexpr float h1[5] = {1.f / 16.f, 1.f / 4.f, 3.f / 8.f, 1.f / 4.f, 1.f / 16.f};
-  const float sn = sigma_n * kLog2e;
+  const float sn = normal_exponent(sigma_n);
   float ws = 0.f, ax = 0.f, ay = 0.f, az = 0.f, av = 0.f;
 #pragma unroll
   for (int dy = -2; dy <= 2; ++dy) {

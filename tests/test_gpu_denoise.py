@@ -123,3 +123,13 @@ def test_denoise_background_at_a_huge_depth(lib):
     got = _run(lib, c, z, n, iterations=1)
     ref_c, ref_v = oden.svgf(c, z, n, iterations=1)
     _check(got, ref_c, ref_v)
+
+
+def test_denoise_largest_normal_exponent(lib):
+    # equal normals weigh 1^sigma_n = 1 however large the exponent, others nothing
+    c, z, n = _image(20, 24, 3)
+    n[...] = [0.0, 0.0, 1.0]
+    n[:, 15:] = [1.0, 0.0, 0.0]
+    got = _run(lib, c, z, n, iterations=2, sigma_n=3e38)
+    ref_c, ref_v = oden.svgf(c, z, n, iterations=2, sigma_n=3e38)
+    _check(got, ref_c, ref_v)
