@@ -59,6 +59,16 @@ __device__ __forceinline__ float neg_ln_series(float d) {
   return fmaf(s * d, d, d);
 }
 
+// Normals that are not of unit length (averaged ones, say) scale all weights of a pixel alike, by about |n|^(2 sigma_n),
+// which leaves the range of a float already for |n|^2 = 1/2.  Both filters form ratios of sums of equal degree in the
+// weights, so the pixel's own normal is divided by |n|^2 where that power is far off 1: its own weight is 1 again.
+template <bool NORMAL>
+__device__ __forceinline__ f3 centre_normal(float4 n4, float sn) {
+  const f3 n = xyz(n4);
+  const float s = dot(n, n);
+  return NORMAL && sn * fabsf(1.0f - s) > 16.0f ? n * __fdividef(1.0f, s) : n;
+}
+
 // Weights w_z w_n w_l of a row of D taps, each one power of two: a[k] is log2(e) times the depth and luminance exponent
 // (>= 0), c[k] = n . n', sn = sigma_n log2(e); NORMAL: sigma_n > 0.  The row takes the series as a whole (one test per
 // row and no divergence on smooth surfaces), or the library logarithm (a normal edge; c <= 0 or NaN: weight 0).
@@ -102,10 +112,10 @@ __device__ __forceinline__ void variance_pixel(int W, int H, int x, int y, const
                                                float sigma_z, float sigma_n, float4* __restrict__ out) {
   const int p = y * W + x;
   const float zp = __ldg(z + p);
-  const f3 np_ = xyz(__ldg(nrm + p));
+  const float sn = normal_exponent(sigma_n);
+  const f3 np_ = centre_normal<NORMAL>(__ldg(nrm + p), sn);
   float inv[49];
   depth_divisors<3>(depth_gradient(z, W, H, x, y), 1.0f, sigma_z, inv);
-  const float sn = normal_exponent(sigma_n);
   float s0 = 0.f, s1 = 0.f, s2 = 0.f;
 #pragma unroll
   for (int dy = -3; dy <= 3; ++dy) {
@@ -174,11 +184,11 @@ __device__ __forceinline__ void atrous_pixel(int W, int H, int step, int x, int 
   const float4 cp = __ldg(in + p);
   const float lp = luminance(cp);
   const float zp = __ldg(z + p);
-  const f3 np_ = xyz(__ldg(nrm + p));
+  const float sn = normal_exponent(sigma_n);
+  const f3 np_ = centre_normal<NORMAL>(__ldg(nrm + p), sn);
   float inv[25];
   depth_divisors<2>(depth_gradient(z, W, H, x, y), (float)step, sigma_z, inv);
   constexpr float h1[5] = {1.f / 16.f, 1.f / 4.f, 3.f / 8.f, 1.f / 4.f, 1.f / 16.f};
-  const float sn = normal_exponent(sigma_n);
   float ws = 0.f, ax = 0.f, ay = 0.f, az = 0.f, av = 0.f;
 #pragma unroll
   for (int dy = -2; dy <= 2; ++dy) {

@@ -133,3 +133,13 @@ def test_denoise_largest_normal_exponent(lib):
     got = _run(lib, c, z, n, iterations=2, sigma_n=3e38)
     ref_c, ref_v = oden.svgf(c, z, n, iterations=2, sigma_n=3e38)
     _check(got, ref_c, ref_v)
+
+
+@pytest.mark.parametrize("length", [0.7, 0.5, 1.3])
+def test_denoise_normals_of_another_length(lib, length):
+    # all weights of a pixel scaled alike, for 0.7 and shorter below the normal range of a float: the same ratios
+    c, z, n = _image(20, 24, 4)
+    n = (n * length).astype(np.float32)
+    got = _run(lib, c, z, n, iterations=2)
+    ref_c, ref_v = oden.svgf(c, z, n, iterations=2)
+    _check(got, ref_c, ref_v)
