@@ -136,3 +136,45 @@ def test_distill_targets(lib, P, K):
     assert (vis[~front] == 0).all() and (depth[~front] == cfg.near).all()
     torch.testing.assert_close(vis[front], tv[front], rtol=0, atol=6e-6)
     torch.testing.assert_close(depth[front], td[front], rtol=0, atol=6e-6)
+
+
+def _sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+# Two warpgroups per SM share the points, so tiles of several pixels need frames sized from the chip: 41 pixels per
+# warpgroup below 16 directions (more in a tile than shared feature slots; at 14 and 15 some tiles have more and some
+# have not, by where they start), 6 above (pixels that start and end anywhere in a tile, or span several).  Against the
+# oracle on rows of the first, a middle and the last warpgroup, and bit for bit in shards, whose tiles fall elsewhere
+@pytest.mark.parametrize("n_dirs, per", [(1, 40), (3, 40), (7, 40), (14, 40), (15, 40), (16, 40), (33, 5), (40, 5),
+                                         (130, 5)])
+def test_frame_tiles_of_several_pixels(lib, n_dirs, per):
+    P = 2 * _sms() * per + 7
+    cfg = helpers.small_cfg(n_dirs=n_dirs, m_dirs=2)
+    sc, gb = helpers.scene_arrays(cfg, 4, bias=0.2, n_pixels=P)
+    r = helpers.renderer_for(cfg, sc)
+    dgb = helpers.to_cuda(gb)
+    out = r.render_frame(dgb, pixel_offset=17).cpu().numpy()
+    lo = 0
+    for hi in (1, P // 3, P // 3 + 2 * _sms() + 1, P):
+        part = {k: v[lo:hi].contiguous() for k, v in dgb.items()}
+        np.testing.assert_array_equal(r.render_frame(part, pixel_offset=17 + lo).cpu().numpy(), out[lo:hi])
+        lo = hi
+    assert r.check() == 0
+    rows = np.r_[0:per + 2, P // 2:P // 2 + per, P - per - 2:P]
+    prm, opt = helpers.oracle_params(sc), helpers.oracle_options(cfg)
+    ref = orender.render(gb, prm, opt, pixel_offset=17, rows=rows)
+    sens = orender.float32_sensitivity(gb, prm, opt, pixel_offset=17, rows=rows, draws=4)
+    ok, stats = helpers.fp32_parity(out[rows, :3], ref, sens)
+    assert ok, stats
+
+
+# three warpgroups per SM: a second and a third tile for some of them, the next tile made while a layer of this one runs;
+# one point's directions (K = 500), tiles of few points, and more points in a tile than slots (K = 1, 3)
+@pytest.mark.parametrize("K, tiles", [(1, 1.01), (3, 2.3), (16, 1.5), (500, 1.01)])
+def test_mlp_rows_second_tiles(lib, K, tiles):
+    test_mlp_rows(lib, int(3 * _sms() * 128 * tiles) // K + 5, K)
+
+
+def test_decode_second_tiles(lib):
+    test_mlp_rows(lib, 2 * 3 * _sms() * 128 + 130, 1)
