@@ -519,9 +519,7 @@ def time_distill(steps: int, warmup: int, barrier, rays: int = 2048, K: int = 10
     ev[0].record(stream)
     dirs = student.distill_dirs(rays, K, 0)
     ev[1].record(stream)
-    feat = teacher.encode(pos)
-    brdf_t = teacher.decode(feat)
-    vis_t, depth_t = teacher.trace(feat, dirs)
+    brdf_t, vis_t, depth_t = d.targets(pos, nrm, dirs)
     ev[2].record(stream)
     student.distill_backward(pos, nrm, dirs, brdf_t, vis_t, depth_t, scratch_loss, *scratch_grads)
     ev[3].record(stream)

@@ -33,12 +33,15 @@ class Distiller:
         self.loss = torch.zeros(3, device=table.device, dtype=torch.float32)
         self.student.set_params(*self.params, env)
 
+    def targets(self, pos: torch.Tensor, normal: torch.Tensor, dirs: torch.Tensor):
+        """The teacher's heads for a batch: B's [P, 8], visibility and depth [P, K]."""
+        feat = self.teacher.encode(pos)
+        return (self.teacher.decode(feat), *self.teacher.distill_targets(feat, dirs, normal))
+
     def step(self, pos: torch.Tensor, normal: torch.Tensor, ray_offset: int = 0) -> torch.Tensor:
         P = pos.shape[0]
         dirs = self.student.distill_dirs(P, self.K, ray_offset)
-        feat = self.teacher.encode(pos)
-        brdf_t = self.teacher.decode(feat)
-        vis_t, depth_t = self.teacher.distill_targets(feat, dirs, normal)
+        brdf_t, vis_t, depth_t = self.targets(pos, normal, dirs)
         for g in self.grads:
             g.zero_()
         self.loss.zero_()

@@ -47,3 +47,9 @@ def test_clock_sampler_parses_clocks_and_throttle_reasons():
     out = cs.stop()
     assert out["sm_mhz"] == 2070.0 and out["sm_max_mhz"] == 2070.0 and out["samples"] == 3
     assert out["reasons"] == ["sw_power_cap"]
+
+
+def test_distill_parts_time_the_steps_own_targets():
+    import inspect
+    src = inspect.getsource(bench.time_distill)
+    assert "d.targets(" in src and "teacher.trace(" not in src and "teacher.decode(" not in src
