@@ -419,7 +419,8 @@ rt_status rt_distill_targets(rt_ctx* ctx, const float* feat, const float* dirs, 
  *             (far - near)| (min-max normalised depth).
  * pos, normal [P][4] (xyz used), dirs [P][K][4] (rt_distill_dirs); brdf_t
  * [P][8] (n', a', r', pad: a teacher's rt_decode), vis_t, depth_t [P][K]
- * (a teacher's rt_trace on dirs).  Sampled directions are constants. */
+ * (a teacher's rt_distill_targets, or rt_trace, on dirs).  Sampled directions
+ * are constants. */
 rt_status rt_distill_backward(rt_ctx* ctx, const float* pos, const float* normal, int64_t P, int32_t K,
                               const float* dirs, const float* brdf_t, const float* vis_t, const float* depth_t,
                               float* loss, float* g_table, float* g_brdf, float* g_irt, void* stream);

@@ -7,9 +7,9 @@
 // times at full magnitude here against 64 times in an FFMA chain.  Measured
 // against 64-bit sums the error is no larger than the chains': 3.4e-5 for both
 // over the stage calls' outputs, and 2.6e-5 to 8.5e-4 against 3.6e-5 to 8.9e-4
-// for whole frames.  The bf16 range is FP32's, so no scaling is needed;
-// infinite operands saturate to the largest finite parts instead of turning
-// the residuals into NaN.
+// for whole frames.  The bf16 range is FP32's, so no scaling is needed.  Parts
+// 0 and 1 saturate, so that an infinite operand does not turn the residuals
+// into NaN; its part 2, the rest, is infinite, and so are its products.
 //
 // Conventions as in tc_common.cuh (a warpgroup owns 128 TMEM lanes, thread t =
 // row t); a split operand in TMEM is three blocks of 32 columns.
@@ -33,7 +33,7 @@ constexpr int HD_IB3 = HD_BW3 + 512;         // [4]
 constexpr int HD_BB3 = HD_IB3 + 4;           // [8]
 constexpr int HD_FLOATS = HD_BB3 + 8;
 
-// bf16 pair, saturating (an infinite value becomes the largest finite one)
+// bf16 pair, rounded; an infinite value becomes the largest finite one
 __device__ __forceinline__ uint32_t pack_bf16_sat(float lo, float hi) {
   uint32_t d;
   asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
