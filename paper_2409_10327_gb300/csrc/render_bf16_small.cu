@@ -4,9 +4,10 @@
 // launch is one chain of evaluations long: 256 points x 32 directions took
 // 40.9 us with 32 valid rows per tile, 20.5 us with four replicas.  Adding the
 // directions' terms in their order in replica 0 (for the bits of a full tile)
-// instead of the replicas' partial sums costs nothing there (20.5 us both) and
-// up to 7 % elsewhere: 256 x 64 under 8 lights 45.0 -> 47.2 us, 256 x 32 with
-// 64 secondary directions 41.1 -> 43.8 us.
+// instead of the replicas' partial sums costs nothing there (cold, 34.0 us both)
+// and up to 7 % elsewhere: 256 x 64 under 8 lights 45.0 -> 47.2 us, 256 x 32
+// with 64 secondary directions 41.1 -> 43.8 us.  One light's terms added a step
+// later, behind the next round trip's barrier: 34.4 us, left out.
 #include "render_bf16_kernel.cuh"
 
 namespace rtk {

@@ -1,7 +1,7 @@
 """BF16 launches too small to fill 128-row tiles share a sample over replica rows: the same frame as in one large launch.
 
-A row computes the same values either way; only the order of the sums over the M secondary and the N primary
-directions differs.  All terms are non-negative, so each sum is within its term count times 2^-23 of the other.
+A row computes the same values either way; for a count of directions that is no multiple of 32 the grouping of the sum
+over them differs.  All terms are non-negative, so each sum is within its term count times 2^-23 of the other.
 """
 import numpy as np
 import pytest
